@@ -9,14 +9,14 @@
 // Variants (padd_chain): XYZZ on one thread (10 multiplications in sequence per
 // mixed addition, with the special-case branches), Edwards on one thread, Edwards
 // on four lanes, and Edwards on four warps (128 threads: each product of an
-// addition on its own warp and spread over that warp's lanes, wpt.cuh). Inputs are
+// addition on its own warp and spread over that warp's lanes, wred.cuh). Inputs are
 // stored points (msm_points_prepare_ex), so the timed kernel is the chain alone.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
 #include "ec.cuh"
 #include "ed.cuh"
-#include "wpt.cuh"
+#include "wred.cuh"
 
 namespace {
 
@@ -106,32 +106,26 @@ __global__ void __launch_bounds__(32) k_chain_ed4(const uint4* __restrict__ pts,
     store_affine_std(out, A);
 }
 
-// Four warps per addition: level 1 {A, B, C} and level 2 {X3, Y3, T3, Z3} on one
-// warp each, every product spread over the lanes of its warp.
+// Four warps per addition: level 1 {e, h, f, g} and level 2 {X3, Y3, T3, Z3} on one
+// warp each, every product spread over the lanes of its warp (wred.cuh).
 __global__ void __launch_bounds__(128, 1) k_chain_edw(const uint4* __restrict__ pts, size_t n, uint32_t* __restrict__ out) {
-    __shared__ __align__(16) uint32_t slots[wpt::kSharedWords];
-    wpt::Group g;
-    wpt::init(g, slots);
-    wpt::ed_set_inf(g);
-    const uint32_t* p = reinterpret_cast<const uint32_t*>(pts);
-    wpt::Operand next = {};
-    if (n) next = wpt::load_operand(p, 3);
+    using C = wred::Edwards;
+    __shared__ __align__(16) int mem[wred::kSharedWords];
+    wred::Group g;
+    wred::init(g, mem);
+    C::set_inf(g);
+    // this warp's coordinate of a stored point (x, y, u = k x y); Z = 1 stays in its slot
+    const int coord = g.w < 3 ? g.w : 0, slot = wred::kQ + (g.w == 2 ? wred::T : g.w);
+    if (g.w == 3) g.st(wred::kQ + wred::Z, wred::unpack(fq::kOne, g.lane));
+    const uint32_t* p = reinterpret_cast<const uint32_t*>(pts) + 12 * coord;
+    int next = n ? wred::unpack(p, g.lane) : 0;
     for (size_t i = 0; i < n; ++i) {
-        const wpt::Operand q = next;    // the next point's loads overlap this addition
-        if (i + 1 < n) next = wpt::load_operand(p + 36 * (i + 1), 3);
-        wpt::ed_madd(g, q);
+        if (g.w < 3) g.st(slot, next);
+        if (i + 1 < n) next = wred::unpack(p + 36 * (i + 1), g.lane);   // overlaps this addition
+        __syncthreads();
+        C::add_op<true>(g);
     }
-    if (threadIdx.x != 0) return;
-    fe c[4];
-    wpt::read_acc(g, c);
-    ed::ext P;
-    P.X = c[0];
-    P.Y = c[1];
-    P.Z = c[2];
-    P.T = c[3];
-    affine A;
-    ed::to_weierstrass(A, P);
-    store_affine_std(out, A);
+    C::store_affine(g, out);
 }
 
 }  // namespace

@@ -40,7 +40,7 @@
 #include "common.cuh"
 #include "ec.cuh"
 #include "ed.cuh"
-#include "wpt.cuh"
+#include "wred.cuh"
 
 namespace {
 
@@ -127,7 +127,6 @@ struct MemQE {
 
 struct ModelXyzz {
     using acc = xyzz;
-    static constexpr int kDblDepth = 3, kAddDepth = 4;  // multiplication levels of dbl4 / add4
     static constexpr int kAccBlocks = 3;  // accumulation blocks of 128 per SM (<= 168 registers)
     static constexpr int kStored = 6;  // affine (x, y)
     static __device__ __forceinline__ void set_inf(acc& P) { ec::set_inf(P); }
@@ -141,29 +140,14 @@ struct ModelXyzz {
     }
     static __device__ __forceinline__ void add_mem(acc& P, const uint4* q) { ec::add_q(P, MemQ{q}); }
     static __device__ __forceinline__ void add(acc& P, const acc& Q) { ec::add(P, Q); }
-    static __device__ __forceinline__ void dbl(acc& P) { ec::dbl(P); }
-    static __device__ __forceinline__ void to_affine(affine& A, const acc& P) { ec::to_affine(A, P); }
-    static __device__ __forceinline__ void dbl4(acc& P, fe* sh, int l) { ec::dbl4(P, sh, l, true); }
     static __device__ __forceinline__ void add4_mem(acc& P, const uint4* q, fe* sh, int l) {
         ec::add4(P, MemQ{q}, sh, l, true);
     }
-    // four-warp group operations (wpt.cuh)
-    static __device__ __forceinline__ void gset_inf(const wpt::Group& g) { wpt::xyzz_set_inf(g); }
-    static __device__ __forceinline__ void gdbl(const wpt::Group& g) { wpt::xyzz_dbl(g); }
-    static __device__ __forceinline__ void gadd(const wpt::Group& g, const wpt::Operand& q) { wpt::xyzz_add(g, q); }
-    static __device__ __forceinline__ void to_affine4(affine& A, const fe (&c)[4]) {
-        xyzz P;
-        P.X = c[0];
-        P.Y = c[1];
-        P.ZZ = c[2];
-        P.ZZZ = c[3];
-        ec::to_affine(A, P);
-    }
+    using chain = wred::Weierstrass;  // four-warp group operations (wred.cuh)
 };
 
 struct ModelEdwards {
     using acc = ed::ext;
-    static constexpr int kDblDepth = 2, kAddDepth = 3;  // multiplication levels of dbl4 / add4
     static constexpr int kAccBlocks = 4;  // accumulation blocks of 128 per SM (<= 128 registers)
     static constexpr int kStored = 9;  // (x, y, u = k x y), the paper's (X, Y, U) with Z = 1
     static __device__ __forceinline__ void set_inf(acc& P) { ed::set_inf(P); }
@@ -195,23 +179,10 @@ struct ModelEdwards {
         ed::add_q(P, MemQE{q});
     }
     static __device__ __forceinline__ void add(acc& P, const acc& Q) { ed::add(P, Q); }
-    static __device__ __forceinline__ void dbl(acc& P) { ed::dbl(P); }
-    static __device__ __forceinline__ void to_affine(affine& A, const acc& P) { ed::to_weierstrass(A, P); }
-    static __device__ __forceinline__ void dbl4(acc& P, fe* sh, int l) { ed::dbl4(P, sh, l, true); }
     static __device__ __forceinline__ void add4_mem(acc& P, const uint4* q, fe* sh, int l) {
         ed::add4(P, MemQE{q}, sh, l, true);
     }
-    static __device__ __forceinline__ void gset_inf(const wpt::Group& g) { wpt::ed_set_inf(g); }
-    static __device__ __forceinline__ void gdbl(const wpt::Group& g) { wpt::ed_dbl(g); }
-    static __device__ __forceinline__ void gadd(const wpt::Group& g, const wpt::Operand& q) { wpt::ed_add(g, q); }
-    static __device__ __forceinline__ void to_affine4(affine& A, const fe (&c)[4]) {
-        ed::ext P;
-        P.X = c[0];
-        P.Y = c[1];
-        P.Z = c[2];
-        P.T = c[3];
-        ed::to_weierstrass(A, P);
-    }
+    using chain = wred::Edwards;
 };
 
 // ---------------------------------------------------------------- stage 1
@@ -1609,66 +1580,61 @@ __global__ void __launch_bounds__(kTreeThreads) k_sum_tree(const uint4* __restri
 
 // ---------------------------------------------------------------- stage 7
 
-// The two latency-bound chains run on one group of four warps per block: each
-// point operation's products are spread over the warps (one product per warp and
-// formula level) and each product over the lanes of its warp (wpt.cuh, wfq.cuh).
-// The next operand's loads are issued before the current operation, so they
-// overlap it.
+// The two latency-bound chains run on one group of four warps per block: each point
+// operation's products are spread over the warps (one product per warp and formula
+// level) and each product over the lanes of its warp (wred.cuh). The next operand's
+// loads are issued before the current operation, so they overlap it.
 
 // Block w: S_w = L sum_{k < logG} 2^k Z_k + Z_logG for window w, by Horner from the
-// top term.
+// top term; S_w is left in the chain's operand form (limbs).
 template <class M>
 __global__ void __launch_bounds__(128, 1) k_window_horner_w(const uint4* __restrict__ Z, int nwin, int logG, int log2L,
-                                                         uint4* __restrict__ S) {
-    __shared__ __align__(16) uint32_t slots[wpt::kSharedWords];
-    wpt::Group g;
-    wpt::init(g, slots);
+                                                         int* __restrict__ S) {
+    using C = typename M::chain;
+    __shared__ __align__(16) int mem[wred::kSharedWords];
     const int w = blockIdx.x;
     if (w >= nwin) return;  // whole block
+    wred::Group g;
+    wred::init(g, mem);
+    C::load_const(g);
     const uint32_t* z = reinterpret_cast<const uint32_t*>(Z + (size_t)w * (logG + 1) * kXyzzVec);
     constexpr size_t kWords = 4 * kXyzzVec;
-    M::gset_inf(g);
-    wpt::Operand next = wpt::load_operand(z + (size_t)(logG > 0 ? logG - 1 : logG) * kWords, 4);
+    C::set_inf(g);
+    wred::Packed next = wred::load_packed(g, z + (size_t)(logG > 0 ? logG - 1 : logG) * kWords);
     for (int k = logG - 1; k >= 0; --k) {
-        const wpt::Operand q = next;   // Z_k
-        next = wpt::load_operand(z + (size_t)(k > 0 ? k - 1 : logG) * kWords, 4);
-        if (k < logG - 1) M::gdbl(g);
-        M::gadd(g, q);
+        const wred::Packed q = next;   // Z_k
+        next = wred::load_packed(g, z + (size_t)(k > 0 ? k - 1 : logG) * kWords);
+        if (k < logG - 1) C::dbl(g, true);
+        C::set_operand(g, q.limb, wred::zero_z(g, q));
+        C::add(g);
     }
-    for (int t = 0; t < log2L; ++t) M::gdbl(g);
-    M::gadd(g, next);                  // Z_logG
-    wpt::store_acc(g, reinterpret_cast<uint32_t*>(S + (size_t)w * kXyzzVec));
+    for (int t = 0; t < log2L; ++t) C::dbl(g, t == log2L - 1);
+    C::set_operand(g, next.limb, wred::zero_z(g, next));   // Z_logG
+    C::add(g);
+    const int v = C::as_operand(g);
+    if (g.lane < 16) S[(size_t)w * wred::kLimbPointWords + 16 * g.w + g.lane] = v;
 }
 
 // sum_w 2^(c w) S_w by Horner over the windows, then the affine result in standard
-// form (thread 0 writes it after the inversion).
+// form.
 template <class M>
-__global__ void __launch_bounds__(128, 1) k_chain_w(const uint4* __restrict__ S, int W, int c, uint32_t* __restrict__ out) {
-    __shared__ __align__(16) uint32_t slots[wpt::kSharedWords];
-    wpt::Group g;
-    wpt::init(g, slots);
-    const uint32_t* s = reinterpret_cast<const uint32_t*>(S);
-    constexpr size_t kWords = 4 * kXyzzVec;
-    M::gset_inf(g);
-    wpt::Operand next = wpt::load_operand(s + (size_t)(W - 1) * kWords, 4);
+__global__ void __launch_bounds__(128, 1) k_chain_w(const int* __restrict__ S, int W, int c, uint32_t* __restrict__ out) {
+    using C = typename M::chain;
+    __shared__ __align__(16) int mem[wred::kSharedWords];
+    wred::Group g;
+    wred::init(g, mem);
+    C::set_inf(g);
+    int next = wred::load_limbs(g, S + (size_t)(W - 1) * wred::kLimbPointWords);
     for (int j = W - 1; j >= 0; --j) {
-        const wpt::Operand q = next;   // S_j
-        if (j > 0) next = wpt::load_operand(s + (size_t)(j - 1) * kWords, 4);
+        g.st(wred::kQ + g.w, next);    // S_j (the operand slots are read before an addition's last barrier)
+        if (j > 0) next = wred::load_limbs(g, S + (size_t)(j - 1) * wred::kLimbPointWords);
         if (j < W - 1)
-            for (int t = 0; t < c; ++t) M::gdbl(g);
-        M::gadd(g, q);
+            for (int t = 0; t < c; ++t) C::dbl(g, t == c - 1);
+        else
+            __syncthreads();
+        C::add(g);
     }
-    if (threadIdx.x != 0) return;
-    fe acc[4];
-    wpt::read_acc(g, acc);
-    affine A;
-    M::to_affine4(A, acc);
-    if (!ec::is_inf(A)) {
-        fq::from_mont(A.x, A.x);
-        fq::from_mont(A.y, A.y);
-    }
-    fq::store(out, A.x);
-    fq::store(out + 12, A.y);
+    C::store_affine(g, out);
 }
 
 // ---------------------------------------------------------------- planning
@@ -1888,7 +1854,7 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool allow_groups = true) {
     const size_t zs = (size_t)p->gw * (p->logG + 1) * p->Q;
     p->off_P0 = take((size_t)p->ngroups * zs * XY);
     p->off_P1 = take((size_t)p->ngroups * zs * XY);
-    p->off_S = take((size_t)p->W * XY);
+    p->off_S = take((size_t)p->W * wred::kLimbPointWords * sizeof(int));
     p->total = off;
     return true;
 }
@@ -2165,7 +2131,7 @@ int enqueue_group_tail_m(const Plan& p, const AccArgs& a, int g, void* workspace
     uint4* V = at<uint4>(workspace, p.off_V) + (size_t)g * yv;
     uint4* P0 = at<uint4>(workspace, p.off_P0) + (size_t)g * zs;
     uint4* P1 = at<uint4>(workspace, p.off_P1) + (size_t)g * zs;
-    uint4* S = at<uint4>(workspace, p.off_S);
+    int* S = at<int>(workspace, p.off_S);
     const size_t nchunks = (size_t)a.nwin * p.cpw;
     // 5. merge partial sums of runs crossing chunk edges (log depth)
     int32_t* start = at<int32_t>(workspace, p.off_start);
@@ -2214,7 +2180,7 @@ int enqueue_group_tail_m(const Plan& p, const AccArgs& a, int g, void* workspace
         zout = tmp;
     }
     // 7a. the per-window sums S_w
-    k_window_horner_w<M><<<(unsigned)a.nwin, 128, 0, s>>>(zin, a.nwin, p.logG, p.log2L, S + (size_t)a.w0 * kXyzzVec);
+    k_window_horner_w<M><<<(unsigned)a.nwin, 128, 0, s>>>(zin, a.nwin, p.logG, p.log2L, S + (size_t)a.w0 * wred::kLimbPointWords);
     note_launches(1);
     return check_launch("msm tail");
 }
@@ -2226,7 +2192,7 @@ int enqueue_group_tail(const Plan& p, const AccArgs& a, int g, void* workspace, 
 
 // 7b. the window combination and normalisation into out.
 int enqueue_chain(const Plan& p, void* workspace, uint32_t* out, cudaStream_t s) {
-    const uint4* S = at<uint4>(workspace, p.off_S);
+    const int* S = at<int>(workspace, p.off_S);
     if (p.edw)
         k_chain_w<ModelEdwards><<<1, 128, 0, s>>>(S, p.W, p.c, out);
     else

@@ -1,8 +1,8 @@
-// Fq arithmetic spread over a warp, for latency-bound chains of point operations.
+// An Fq multiplication spread over a warp on canonical 32-bit limbs (a variant of
+// fq_mul_batch_variant; the chains of point operations use the redundant limbs of wred.cuh).
 //
 // A field element is held by a whole warp: lane j < 12 holds limb j, lanes 12..31
-// hold 0. Values are in Montgomery form (x 2^384 mod p), in [0, 2p) as in fq.cuh,
-// or a few multiples of p for the unfolded add / subtract that feed products.
+// hold 0. Values are in Montgomery form (x 2^384 mod p), in [0, 2p) as in fq.cuh.
 //
 // Multiplication (Montgomery, R = 2^384) takes three column products instead of
 // twelve sequential rows:
@@ -14,7 +14,7 @@
 // fetched per lane by shuffles (the operand b) or, for the constants p' and p of
 // the two reduction products, kept per lane in registers -- so the twelve rows run
 // in parallel across lanes and a product costs about thirty shared-memory and
-// shuffle operations, the resource the four warps of a group share. The column sums (below 2^37) are then turned into words
+// shuffle operations. The column sums (below 2^37) are then turned into words
 // in constant time: after adding the previous column's high part, each lane
 // either generates a carry, propagates one (its word is 2^32 - 1) or neither; with
 // G and P the warp's ballots of those flags, the carries into the lanes are the
@@ -42,11 +42,11 @@ __device__ __forceinline__ int lane() { return threadIdx.x & 31; }
 // operand, T mod R and the quotient m (12 words each, 16-byte aligned).
 constexpr int kScratchWords = 36;
 
-// Per-lane values: limb `lane` of p, 2p and 4p, the column operands p_{lane - d} and
+// Per-lane values: limb `lane` of p, the column operands p_{lane - d} and
 // p'_{lane - d} for d = 0..12 (0 outside the twelve limbs), and the shared-memory
 // address of this warp's scratch.
 struct Consts {
-    uint32_t p, p2, p4, p6;
+    uint32_t p;
     uint32_t pc[13], qc[13];
     uint32_t scratch;
 };
@@ -63,15 +63,7 @@ __device__ __forceinline__ uint32_t keep12(uint32_t v);
 __device__ __forceinline__ void init(Consts& K, uint32_t* scratch) {
     const int l = lane();
     K.p = limb_of(fq::kP);
-    K.p2 = limb_of(fq::k2P);
     const uint32_t q = limb_of(kPInvNeg);
-    // 4p = 2 (2p): limbs of 2p shifted left by one bit across lanes
-    const uint32_t below = __shfl_up_sync(kFull, K.p2, 1);
-    K.p4 = l < 12 ? (K.p2 << 1) | (l ? below >> 31 : 0u) : 0u;
-    {   // 6p = 4p + 2p
-        const uint32_t s = K.p4 + K.p2;
-        K.p6 = keep12(normalize(s, (uint32_t)(s < K.p4)));
-    }
 #pragma unroll
     for (int d = 0; d < 13; ++d) {
         K.pc[d] = __shfl_sync(kFull, K.p, (l - d) & 31);   // negative sources wrap to lanes >= 20: zero
@@ -156,82 +148,12 @@ __device__ __forceinline__ uint32_t mul(uint32_t a, uint32_t b, const Consts& K)
     return keep12(__shfl_down_sync(kFull, u, 12));  // (T + m p) / R
 }
 
-// a + b (no reduction; for values that feed products).
-__device__ __forceinline__ uint32_t add_nr(uint32_t a, uint32_t b) {
-    const uint32_t s = a + b;
-    return keep12(normalize(s, (uint32_t)(s < a)));
-}
-
-// a - b + K p with K p given per lane (kp = K.p2 or K.p4): a + kp + (2^384 - 1 - b) + 1
-// taken mod 2^384 (needs b <= a + K p).
-__device__ __forceinline__ uint32_t sub_kp(uint32_t a, uint32_t b, uint32_t kp) {
-    const int l = lane();
-    const uint64_t v = (uint64_t)a + kp + (l < 12 ? ~b : 0u) + (l == 0 ? 1u : 0u);
-    return keep12(normalize((uint32_t)v, (uint32_t)(v >> 32)));
-}
-
-// sum of the P positive terms - sum of the Q negative terms + k p (kp = k p's limb
-// `lane`), with one carry resolution: each subtraction is a two's complement over
-// the twelve limbs, so the per-lane sum stays below 2^35 and its high part flows up.
-// Needs the result to be non-negative (the caller's k p covers the negative terms).
-template <int P, int Q>
-__device__ __forceinline__ uint32_t lincomb(const uint32_t (&pos)[P], const uint32_t (&neg)[Q], uint32_t kp) {
-    const int l = lane();
-    uint64_t v = (uint64_t)kp + (l == 0 ? (uint32_t)Q : 0u);
-#pragma unroll
-    for (int i = 0; i < P; ++i) v += pos[i];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) v += l < 12 ? ~neg[i] : 0u;
-    return keep12(normalize((uint32_t)v, (uint32_t)(v >> 32)));
-}
-
-__device__ __forceinline__ uint32_t sub_nr2(uint32_t a, uint32_t b, const Consts& K) { return sub_kp(a, b, K.p2); }
-__device__ __forceinline__ uint32_t sub_nr4(uint32_t a, uint32_t b, const Consts& K) { return sub_kp(a, b, K.p4); }
-
-// Folded forms for [0, 2p) operands and results. The two candidates are formed in
-// parallel; word 12 of the 13-word sum says which one is in range.
-__device__ __forceinline__ uint32_t add(uint32_t a, uint32_t b, const Consts& K) {
-    const int l = lane();
-    const uint32_t s = a + b;
-    const uint32_t sum = normalize(s, (uint32_t)(s < a));                 // a + b
-    const uint64_t v = (uint64_t)a + b + (l < 12 ? ~K.p2 : 0u) + (l == 0 ? 1u : 0u);
-    const uint32_t red = normalize((uint32_t)v, (uint32_t)(v >> 32));    // a + b - 2p + 2^384
-    const bool ge = __shfl_sync(kFull, red, 12) != 0;                     // a + b >= 2p
-    return keep12(ge ? red : sum);
-}
-
-__device__ __forceinline__ uint32_t sub(uint32_t a, uint32_t b, const Consts& K) {
-    const int l = lane();
-    const uint64_t v = (uint64_t)a + (l < 12 ? ~b : 0u) + (l == 0 ? 1u : 0u);
-    const uint32_t d = normalize((uint32_t)v, (uint32_t)(v >> 32));      // a - b + 2^384
-    const uint32_t e = sub_kp(a, b, K.p2);                                // a - b + 2p
-    const bool ge = __shfl_sync(kFull, d, 12) != 0;                       // a >= b
-    return keep12(ge ? d : e);
-}
-
 // [0, 2p) -> [0, p).
 __device__ __forceinline__ uint32_t canon(uint32_t x, const Consts& K) {
     const int l = lane();
     const uint64_t v = (uint64_t)x + (l < 12 ? ~K.p : 0u) + (l == 0 ? 1u : 0u);
     const uint32_t d = normalize((uint32_t)v, (uint32_t)(v >> 32));      // x - p + 2^384
     return keep12(__shfl_sync(kFull, d, 12) != 0 ? d : x);
-}
-
-// x in [0, 2p) is zero mod p (x = 0 or x = p); the same answer in every lane.
-__device__ __forceinline__ bool is_zero(uint32_t x, const Consts& K) {
-    const int l = lane();
-    const uint32_t nz = __ballot_sync(kFull, l < 12 && x != 0u);
-    const uint32_t np = __ballot_sync(kFull, l < 12 && x != K.p);
-    return nz == 0u || np == 0u;
-}
-
-// Every limb zero (a raw all-zero value in memory).
-__device__ __forceinline__ bool is_zero_raw(uint32_t x) { return __ballot_sync(kFull, lane() < 12 && x != 0u) == 0u; }
-
-// A 12-word slot (shared or global memory): lane j < 12 takes word j.
-__device__ __forceinline__ uint32_t load(const uint32_t* slot) { return lane() < 12 ? slot[lane()] : 0u; }
-__device__ __forceinline__ void store(uint32_t* slot, uint32_t v) {
-    if (lane() < 12) slot[lane()] = v;
 }
 
 }  // namespace wfq
