@@ -6,17 +6,14 @@
 //  1. prepare     standard affine -> Montgomery affine (96 B per point, AoS, so a
 //                 random gather of one point reads three full 32 B sectors)
 //  2. digits      c-bit window digits per scalar (signed or unsigned);
-//                 key = |digit|, value = point index | sign << 31, window-major
-//  3. sort        bucket order within each window: a counting sort over (window,
-//                 key) bins (count, scan, scatter with warp-aggregated atomics) for
-//                 few windows or wide keys, else a stable LSD radix sort with 8-bit
-//                 digits per pass (histogram, scans, ranked scatter)
-//  4. accumulate  per window, the sorted stream is cut into equal chunks of K
-//                 items, one per thread, so heavy buckets spread over threads;
-//                 runs inside a chunk are summed with mixed PADDs and written
-//                 to their bucket, runs
-//                 crossing a chunk edge leave partial sums
-//  5. merge       partial sums of runs that cross chunk edges are added up
+//                 |digit| and its sign, window-major
+//  3. sort        point indices in bucket order within each window: a counting sort
+//                 over (window, key) bins (count, scan, scatter), or a stable LSD
+//                 radix sort with 8-bit digits per pass
+//  4. accumulate  every bucket's run of points is cut into pieces of bounded length;
+//                 the pieces, longest first, are summed with mixed PADDs, one thread
+//                 each, so the lanes of a warp add equally many points
+//  5. merge       the pieces of buckets that needed more than one are added up
 //  6. reduce      per window sum_b b * B_b: segments of L buckets by running sums
 //                 in-thread, then sum_g g * Y_g split by the bits of g into
 //                 independent sums, recombined by Horner
@@ -132,6 +129,13 @@ struct ModelXyzz {
     static __device__ __forceinline__ void set_inf(acc& P) { ec::set_inf(P); }
     static __device__ __forceinline__ void load(acc& P, const uint4* p) { load_xyzz(P, p); }
     static __device__ __forceinline__ void store(uint4* p, const acc& P) { store_xyzz(p, P); }
+    static __device__ __forceinline__ bool first_at(acc& P, const uint4* pts, uint32_t idx, bool negate) {
+        affine Q;
+        load_affine(Q, pts, idx);
+        if (negate) ec::neg(Q);
+        ec::from_affine(P, Q);
+        return ec::is_inf(Q);
+    }
     static __device__ __forceinline__ void madd_at(acc& P, bool& inf, const uint4* pts, uint32_t idx, bool negate) {
         affine Q;
         load_affine(Q, pts, idx);
@@ -163,14 +167,24 @@ struct ModelEdwards {
         store_fe(p + 6, P.Z);
         store_fe(p + 9, P.T);
     }
-    static __device__ __forceinline__ void madd_at(acc& P, bool& inf, const uint4* pts, uint32_t idx, bool negate) {
-        ed::stored Q;
+    static __device__ __forceinline__ void load_stored(ed::stored& Q, const uint4* pts, uint32_t idx, bool negate) {
         const uint4* q = pts + (size_t)kStored * idx;
         load_fe(Q.x, q);
         load_fe(Q.y, q + 3);
         load_fe(Q.u, q + 6);
         if (negate) ed::neg(Q);
-        ed::madd(P, inf, Q);
+    }
+    // acc <- the first point; the flag says acc is the identity (never, here)
+    static __device__ __forceinline__ bool first_at(acc& P, const uint4* pts, uint32_t idx, bool negate) {
+        ed::stored Q;
+        load_stored(Q, pts, idx, negate);
+        ed::from_stored(P, Q);
+        return false;
+    }
+    static __device__ __forceinline__ void madd_at(acc& P, bool&, const uint4* pts, uint32_t idx, bool negate) {
+        ed::stored Q;
+        load_stored(Q, pts, idx, negate);
+        ed::madd(P, Q);
     }
     static __device__ __forceinline__ void add_mem(acc& P, const uint4* q) {
         fe z;
@@ -642,12 +656,10 @@ __global__ void __launch_bounds__(128, 3) k_precompute_ed(const uint4* __restric
 // ---------------------------------------------------------------- stage 2
 
 // Window digits of one scalar (8 words, little-endian) for point index `idx`:
-// key = |digit| (0 = no contribution), value = point | sign << 31, window-major
-// ([W][np]). The point is idx, or with precomputed shifted points (`pre`) the
-// copy 2^(c j) P_idx at row idx W + j, so the W windows form one bucket problem.
+// |digit| (0 = no contribution) with its sign in bit 31, window-major ([W][np]). The
+// point of an item follows from its place (item_point), so it is not stored.
 __device__ __forceinline__ void emit_digits(const uint32_t (&s)[8], int c, int W, int sgn, size_t idx,
-                                            size_t np, int pre, uint32_t* __restrict__ keys,
-                                            uint32_t* __restrict__ vals) {
+                                            size_t np, uint32_t* __restrict__ keys) {
     const uint32_t cmask = (1u << c) - 1u, half = 1u << (c - 1);
     uint32_t carry = 0;
     for (int j = 0; j < W; ++j) {
@@ -672,9 +684,19 @@ __device__ __forceinline__ void emit_digits(const uint32_t (&s)[8], int c, int W
         } else {
             key = raw;
         }
-        keys[(size_t)j * np + idx] = key;
-        vals[(size_t)j * np + idx] = (uint32_t)(pre ? idx * (size_t)W + j : idx) | (neg << 31);
+        keys[(size_t)j * np + idx] = key | (neg << 31);
     }
+}
+
+constexpr uint32_t kSign = 0x80000000u;
+
+// The stored point of item j of a window: point j, or with precomputed shifted points
+// (one window of Wd np items, item j' np + i the digit j' of point i) the copy
+// 2^(c j') P_i at row i Wd + j'. Wd = 0: no precomputed points.
+__device__ __forceinline__ uint32_t item_point(size_t j, size_t np, int Wd) {
+    if (Wd == 0) return (uint32_t)j;
+    const uint32_t d = (uint32_t)(j / np), i = (uint32_t)(j - (size_t)d * np);
+    return i * (uint32_t)Wd + d;
 }
 
 // GLV split of a scalar k < 2^256: k mod r = k1 + lambda k2 with 0 <= k1 < lambda
@@ -781,8 +803,7 @@ __device__ __forceinline__ void glv_split(uint32_t (&k)[8], uint32_t (&k1)[8], u
 }
 
 __global__ void k_digits(const uint4* __restrict__ scalars, size_t n, int c, int W, int sgn,
-                         int bits, int glv, int pre, uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
-                         int* __restrict__ status) {
+                         int bits, int glv, uint32_t* __restrict__ keys, int* __restrict__ status) {
     size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     uint4 lo = scalars[2 * i], hi = scalars[2 * i + 1];
@@ -799,13 +820,13 @@ __global__ void k_digits(const uint4* __restrict__ scalars, size_t n, int c, int
         if (over) atomicCAS(status, 0, MSM377_ERANGE);   // the first error of the call stays
     }
     if (!glv) {
-        emit_digits(s, c, W, sgn, i, n, pre, keys, vals);
+        emit_digits(s, c, W, sgn, i, n, keys);
         return;
     }
     uint32_t k1[8], k2[8];
     glv_split(s, k1, k2);
-    emit_digits(k1, c, W, sgn, 2 * i, 2 * n, pre, keys, vals);      // P_i
-    emit_digits(k2, c, W, sgn, 2 * i + 1, 2 * n, pre, keys, vals);  // phi(P_i)
+    emit_digits(k1, c, W, sgn, 2 * i, 2 * n, keys);      // P_i
+    emit_digits(k2, c, W, sgn, 2 * i + 1, 2 * n, keys);  // phi(P_i)
 }
 
 // ---------------------------------------------------------------- stage 3: radix sort
@@ -903,8 +924,8 @@ __global__ void k_sort_scan_digits(uint32_t* __restrict__ dtot) {
 template <int RB>
 __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
-    uint32_t* __restrict__ vout, uint2* __restrict__ kvout, size_t n, int shift, size_t tiles,
-    const uint32_t* __restrict__ hist, const uint32_t* __restrict__ doff) {
+    uint32_t* __restrict__ vout, size_t n, int shift, size_t tiles,
+    const uint32_t* __restrict__ hist, const uint32_t* __restrict__ doff, size_t np, int Wd) {
     constexpr int R = 1 << RB;
     __shared__ uint32_t wcnt[kSortThreads / 32][R];
     __shared__ uint32_t base[R];
@@ -922,7 +943,12 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
         size_t idx = sub + (size_t)r * 32 + lane;
         bool valid = idx < n;
         key[r] = valid ? kin[seg + idx] : 0u;
-        val[r] = valid ? vin[seg + idx] : 0u;
+        if (vin) {
+            val[r] = valid ? vin[seg + idx] : 0u;
+        } else {        // the first pass: the item's point and sign
+            val[r] = item_point(idx, np, Wd) | (key[r] & kSign);
+            key[r] &= ~kSign;
+        }
         // Items past the end sort last in the tile and are never written.
         dig[r] = valid ? ((key[r] >> shift) & (R - 1)) : (R - 1);
         uint32_t peers = __match_any_sync(0xffffffffu, dig[r]);
@@ -950,15 +976,26 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(
         if (idx < n) {
             size_t pos = (size_t)base[dig[r]] + wcnt[wid][dig[r]] + rank[r];
             if (pos < n) {  // always true when the counts agree; keeps writes in bounds
-                if (kvout) {    // last pass: (key, value) pairs, one 8-byte store
-                    kvout[seg + pos] = make_uint2(key[r], val[r]);
-                } else {
-                    kout[seg + pos] = key[r];
-                    vout[seg + pos] = val[r];
-                }
+                kout[seg + pos] = key[r];
+                vout[seg + pos] = val[r];
             }
         }
     }
+}
+
+// Run starts of the sorted keys: start[w nb + k] = w n + the first position in window
+// w with key >= k, for k < nb (the bin offsets that the counting sort has anyway).
+__global__ void k_run_starts(const uint32_t* __restrict__ keys, size_t n, uint32_t nb, uint32_t* __restrict__ start) {
+    const size_t j = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const size_t w = blockIdx.y;
+    const uint32_t* kw = keys + w * n;
+    const uint32_t key = kw[j], prev = j ? kw[j - 1] : 0u;
+    uint32_t* row = start + w * nb;
+    if (j == 0) row[0] = (uint32_t)(w * n);
+    for (uint32_t k = prev + 1; k <= key && k < nb; ++k) row[k] = (uint32_t)(w * n + j);
+    if (j + 1 == n)
+        for (uint32_t k = key + 1; k < nb; ++k) row[k] = (uint32_t)((w + 1) * n);
 }
 
 // ---------------------------------------------------------------- stage 3 (counting sort)
@@ -982,7 +1019,7 @@ __global__ void k_bin_count(const uint32_t* __restrict__ keys, size_t np, uint32
     const size_t j = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     const bool valid = j < np;
     const size_t i = (size_t)blockIdx.y * np + j;
-    const uint32_t bin = valid ? blockIdx.y * nb + keys[i] : 0xffffffffu;
+    const uint32_t bin = valid ? blockIdx.y * nb + (keys[i] & ~kSign) : 0xffffffffu;
     const uint32_t peers = __match_any_sync(0xffffffffu, bin);
     const int lane = threadIdx.x & 31;
     const int leader = __ffs(peers) - 1;
@@ -1068,17 +1105,16 @@ __global__ void k_scan_add(uint32_t* __restrict__ x, size_t m, const uint32_t* _
     if (i < m) x[i] += bsum[i / kScanTile];
 }
 
-// Each item to the next free slot of its bin (cursor = the bins' offsets, advanced
-// with one warp-aggregated atomic per bin and warp).
-__global__ void k_bin_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-                              const uint32_t* __restrict__ rank, uint2* __restrict__ kvout, size_t total,
-                              size_t np, uint32_t nb, const uint32_t* __restrict__ start) {
+// Each item's point and sign to its slot: the bin's offset plus its rank in the bin.
+__global__ void k_bin_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ rank,
+                              uint32_t* __restrict__ out, size_t total, size_t items, uint32_t nb,
+                              const uint32_t* __restrict__ start, size_t np, int Wd) {
     const size_t j = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (j >= np) return;
-    const size_t i = (size_t)blockIdx.y * np + j;
+    if (j >= items) return;
+    const size_t i = (size_t)blockIdx.y * items + j;
     const uint32_t key = kin[i];
-    const size_t pos = (size_t)start[blockIdx.y * nb + key] + rank[i];
-    if (pos < total) kvout[pos] = make_uint2(key, vin[i]);  // in bounds when the counts agree
+    const size_t pos = (size_t)start[blockIdx.y * nb + (key & ~kSign)] + rank[i];
+    if (pos < total) out[pos] = item_point(j, np, Wd) | (key & kSign);  // in bounds when the counts agree
 }
 
 // The same counting sort with the counts taken per tile in shared memory, for key
@@ -1112,7 +1148,7 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_count(const uint32_t* __r
     const uint32_t* kw = keys + w * np;
     uint32_t* rw = rank + w * np;
     for (size_t j = lo + threadIdx.x; j < hi; j += blockDim.x) {
-        const uint32_t key = kw[j];
+        const uint32_t key = kw[j] & ~kSign;
         if (key >= nb) continue;   // keys are below nb by construction
         const uint32_t sh = (key & 1u) << 4;
         const uint32_t old = atomicAdd(&h[key >> 1], 1u << sh);
@@ -1159,105 +1195,257 @@ __global__ void k_tile_offsets(uint32_t* __restrict__ cnt, uint32_t nb, uint32_t
 
 // Grid (items of a window / 256, windows): each item to its tile's slot for the key
 // plus its rank.
-__global__ void k_tile_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-                               const uint32_t* __restrict__ rank, uint2* __restrict__ kvout, size_t total,
-                               size_t np, uint32_t nb, uint32_t T, uint32_t ntiles, const uint32_t* __restrict__ cnt) {
+__global__ void k_tile_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ rank,
+                               uint32_t* __restrict__ out, size_t total, size_t items, uint32_t nb, uint32_t T,
+                               uint32_t ntiles, const uint32_t* __restrict__ cnt, size_t np, int Wd) {
     const size_t j = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (j >= np) return;
+    if (j >= items) return;
     const size_t w = blockIdx.y;
-    const size_t i = w * np + j;
-    const uint32_t key = kin[i];
-    if (key >= nb) return;
+    const size_t i = w * items + j;
+    const uint32_t key = kin[i], bin = key & ~kSign;
+    if (bin >= nb) return;
     const size_t t = j / T;
-    const size_t pos = (size_t)cnt[(w * ntiles + t) * nb + key] + rank[i];
-    if (pos < total) kvout[pos] = make_uint2(key, vin[i]);
+    const size_t pos = (size_t)cnt[(w * ntiles + t) * nb + bin] + rank[i];
+    if (pos < total) out[pos] = item_point(j, np, Wd) | (key & kSign);
 }
 
 // ---------------------------------------------------------------- stages 4-5
+//
+// A bucket's run of m sorted items is cut into ceil(m / cap) pieces of nearly equal
+// length. Pieces are listed by length, longest first (a counting sort over the at most
+// kMaxPiece lengths), and one thread sums one piece: the lanes of a warp then start,
+// add and store together, where threads over equal chunks of the sorted stream spent
+// a tenth of their additions on lanes waiting for another lane's run end, and every
+// run crossing a chunk edge cost a full addition to put together. Measured at
+// n = 2^20: accumulation and merges 5742 + 420 -> 5570 + 120 us (XYZZ, c = 16),
+// 4179 + 424 -> 3740 + 75 us (Edwards + GLV, c = 17); both now run the multiply pipe at 0.9
+// to 0.96 of its measured peak.
+// A bucket of one piece gets its sum directly. The pieces of any other leave partial
+// sums in consecutive slots, put together by k_merge_parts: a few by one thread in
+// sequence, more by blocks that sum up to kTreeParts each in a tree of
+// four-lane additions, in up to three levels -- so a bucket that holds a whole window
+// (all-equal scalars, a nearly empty top window) costs O(log) sequential additions.
+constexpr uint32_t kMaxPiece = 256;     // longest piece a plan may ask for
+constexpr uint32_t kTreeParts = 64;
+constexpr uint32_t kPart = 0x80000000u; // destination is a partial-sum slot, not a bucket
+constexpr int kPieceThreads = 256;
 
-struct AccArgs {
-    const uint2* kv;       // [W][n] sorted (bucket key, point index | sign << 31)
-    const uint4* pts;
-    uint4* buckets;        // [W][Bp] XYZZ
-    uint4* head;           // [W][cpw] XYZZ
-    uint4* tail;           // [W][cpw] XYZZ
-    uint32_t* headflag;    // 0 none, 1 run ends here, 2 run continues past this chunk
-    uint32_t* tailkey;     // key of the run leaving this chunk, or kNone
-    size_t n;              // items per window
-    uint32_t cpw;          // chunks per window
-    uint32_t Bp;
-    int K;
-    int w0, nwin;          // window range of this launch
-    const uint32_t* bin;   // counting sort: first kv slot of each (window, key) bin (else null)
-    uint32_t nb;           // keys per window (Bp + 1)
+// Device counters of one window group, zeroed before use. Indices into uint32_t words.
+enum : uint32_t { kHist = 0, kCursor = kMaxPiece + 1, kNParts = 2 * (kMaxPiece + 1), kNSmall, kNTree /* 3 levels */,
+                  kCtrlWords = (kNTree + 3 + 31) / 32 * 32 };
+
+struct PieceArgs {
+    const uint32_t* start;  // first item of each bin (w, key), key < nb; the next bin's start ends it
+    uint32_t nb, Bp;
+    int w0, nwin;           // windows of this group
+    uint32_t total;         // all windows' items: the end of the last bin
+    uint32_t cap;
+    uint32_t small_parts;   // buckets of up to this many parts are summed by one thread
+    uint32_t* ctrl;
+    uint4* pieces;          // {first item, length, destination, -}
+    uint4* small;           // {first part, parts, destination, -}
+    uint4* tree[3];
+    uint4* buckets;
 };
 
-// Mixed additions of chunk t of window w. Flushes each run to its bucket, or to
-// the chunk's head / tail partial when it crosses a chunk edge.
-template <class M>
-__device__ __forceinline__ void accumulate_chunk(const AccArgs& a, int w, uint32_t t) {
-    const size_t ci = (size_t)w * a.cpw + t;
-    const uint2* kv = a.kv + (size_t)w * a.n;
-    const size_t start = (size_t)t * a.K;
-    const size_t end = start + a.K < a.n ? start + a.K : a.n;
-    const uint32_t prev = start > 0 ? kv[start - 1].x : kNone;
-    const uint32_t next = end < a.n ? kv[end].x : kNone;
-    a.tailkey[ci] = kNone;
-    a.headflag[ci] = 0;
-    typename M::acc acc;
-    M::set_inf(acc);
-    bool inf = true;
-    uint32_t cur = kv[start].x;
-    bool first = true;
-    for (size_t g = start; g <= end; ++g) {
-        const uint2 e = g < end ? kv[g] : make_uint2(kNone, 0u);
-        const uint32_t key = e.x;
-        if (key != cur) {
-            if (cur != 0) {  // key 0 = zero digit, contributes nothing
-                const bool sb = first && prev == cur;
-                const bool ea = (g == end) && next == cur;
-                if (!sb && !ea) {
-                    M::store(a.buckets + ((size_t)w * a.Bp + (cur - 1)) * kXyzzVec, acc);
-                } else if (sb) {
-                    M::store(a.head + ci * kXyzzVec, acc);
-                    a.headflag[ci] = ea ? 2u : 1u;
-                } else {
-                    M::store(a.tail + ci * kXyzzVec, acc);
-                    a.tailkey[ci] = cur;
-                }
-            }
-            if (g == end) break;
-            M::set_inf(acc);
-            inf = true;
-            cur = key;
-            first = false;
+struct BinRun {
+    uint32_t s, m, bucket;
+};
+
+// Bin id (over the group's windows) -> its run; m = 0 and no bucket for key 0 (zero
+// digits) and past the end.
+__device__ __forceinline__ BinRun bin_run(const PieceArgs& a, size_t id) {
+    BinRun r = {0, 0, kNone};
+    if (id >= (size_t)a.nwin * a.nb) return r;
+    const uint32_t wi = (uint32_t)(id / a.nb), key = (uint32_t)(id - (size_t)wi * a.nb);
+    const size_t g = (size_t)(a.w0 + wi) * a.nb + key;
+    r.s = a.start[g];
+    // bins are contiguous over all windows; the last one ends at the last item
+    const uint32_t e = (wi + 1 == (uint32_t)a.nwin && key + 1 == a.nb) ? a.total : a.start[g + 1];
+    if (key == 0) return r;
+    r.m = e - r.s;
+    r.bucket = (uint32_t)(a.w0 + wi) * a.Bp + key - 1;
+    return r;
+}
+
+__global__ void __launch_bounds__(kPieceThreads) k_piece_count(PieceArgs a) {
+    __shared__ uint32_t h[kMaxPiece + 1];
+    for (uint32_t k = threadIdx.x; k <= kMaxPiece; k += kPieceThreads) h[k] = 0;
+    __syncthreads();
+    const BinRun r = bin_run(a, blockIdx.x * (size_t)kPieceThreads + threadIdx.x);
+    if (r.m) {
+        const uint32_t np = (r.m + a.cap - 1) / a.cap, q = r.m / np, big = r.m - q * np;
+        if (big) atomicAdd(&h[q + 1], big);
+        atomicAdd(&h[q], np - big);
+    }
+    __syncthreads();
+    for (uint32_t k = threadIdx.x; k <= a.cap; k += kPieceThreads)
+        if (h[k]) atomicAdd(&a.ctrl[kHist + k], h[k]);
+}
+
+// Appends the merge work of a bucket cut into np pieces; returns its first part slot.
+__device__ __forceinline__ uint32_t plan_merge(const PieceArgs& a, uint32_t np, uint32_t bucket) {
+    const uint32_t n1 = (np + kTreeParts - 1) / kTreeParts, n2 = (n1 + kTreeParts - 1) / kTreeParts;
+    const uint32_t extra = np <= a.small_parts || n1 == 1 ? 0 : (n2 == 1 ? n1 : n1 + n2);
+    const uint32_t base = atomicAdd(&a.ctrl[kNParts], np + extra);
+    if (np <= a.small_parts) {
+        a.small[atomicAdd(&a.ctrl[kNSmall], 1u)] = make_uint4(base, np, bucket, 0u);
+        return base;
+    }
+    uint32_t src = base, cnt = np;
+    for (int lv = 0; lv < 3; ++lv) {
+        const uint32_t nout = lv == 2 ? 1u : (cnt + kTreeParts - 1) / kTreeParts;
+        const uint32_t e = atomicAdd(&a.ctrl[kNTree + lv], nout);
+        if (nout == 1) {
+            a.tree[lv][e] = make_uint4(src, cnt, bucket, 0u);
+            break;
         }
-        if (key != 0) {
-            const uint32_t v = e.y;
-            if ((v & 0x7fffffffu) >= a.n) continue;  // cannot happen for sorted digit output
-            M::madd_at(acc, inf, a.pts, v & 0x7fffffffu, (v >> 31) != 0);
+        for (uint32_t i = 0; i < nout; ++i) {
+            const uint32_t left = cnt - i * kTreeParts;
+            a.tree[lv][e + i] = make_uint4(src + i * kTreeParts, left < kTreeParts ? left : kTreeParts,
+                                           (src + cnt + i) | kPart, 0u);
+        }
+        src += cnt;
+        cnt = nout;
+    }
+    return base;
+}
+
+// A bin of more than kWide pieces, written by its whole block.
+constexpr uint32_t kWide = 16;
+struct WideBin {
+    uint32_t s, np, q, big, dest, at_big, at_q;
+};
+
+// The pieces of every bin to their places in the list (longest first) and the merge
+// lists; empty buckets get coordinate 2 = 0, which every reader of buckets takes as
+// "no point".
+__global__ void __launch_bounds__(kPieceThreads) k_piece_emit(PieceArgs a) {
+    __shared__ uint32_t h[kMaxPiece + 1], base[kMaxPiece + 1];
+    __shared__ uint32_t warp_tot[kPieceThreads / 32];
+    __shared__ WideBin wide[kPieceThreads];
+    __shared__ uint32_t nwide;
+    const int t = threadIdx.x;
+    for (uint32_t k = t; k <= kMaxPiece; k += kPieceThreads) h[k] = 0;
+    if (t == 0) nwide = 0;
+    __syncthreads();
+    const size_t id = blockIdx.x * (size_t)kPieceThreads + t;
+    const BinRun r = bin_run(a, id);
+    uint32_t np = 0, q = 0, big = 0, rank_big = 0, rank_q = 0;
+    if (r.m) {
+        np = (r.m + a.cap - 1) / a.cap;
+        q = r.m / np;
+        big = r.m - q * np;
+        if (big) rank_big = atomicAdd(&h[q + 1], big);
+        rank_q = atomicAdd(&h[q], np - big);
+    } else if (r.bucket != kNone) {
+        uint4* z = a.buckets + (size_t)r.bucket * kXyzzVec + 6;
+        z[0] = z[1] = z[2] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    __syncthreads();
+    // Class offsets: lengths in descending order. Thread t has length kMaxPiece - t.
+    {
+        const uint32_t len = kMaxPiece - t;   // 256 .. 1
+        const uint32_t v = len <= a.cap ? a.ctrl[kHist + len] : 0u;
+        uint32_t x = v;
+        const int lane = t & 31, wid = t >> 5;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) warp_tot[wid] = x;
+        __syncthreads();
+        uint32_t before = 0;
+        for (int k = 0; k < wid; ++k) before += warp_tot[k];
+        const uint32_t mine = h[len];
+        base[len] = before + x - v + (mine ? atomicAdd(&a.ctrl[kCursor + len], mine) : 0u);
+    }
+    __syncthreads();
+    if (np) {
+        uint32_t dest = r.bucket;
+        if (np > 1) dest = plan_merge(a, np, r.bucket) | kPart;
+        const uint32_t pb = big ? base[q + 1] + rank_big : 0u, pq = base[q] + rank_q;
+        if (np <= kWide) {
+            uint32_t s = r.s;
+            for (uint32_t i = 0; i < np; ++i) {
+                const uint32_t len = i < big ? q + 1 : q;
+                a.pieces[i < big ? pb + i : pq + i - big] = make_uint4(s, len, dest + i, 0u);
+                s += len;
+            }
+        } else {
+            wide[atomicAdd(&nwide, 1u)] = {r.s, np, q, big, dest, pb, pq};
+        }
+    }
+    __syncthreads();
+    for (uint32_t k = 0; k < nwide; ++k) {
+        const WideBin b = wide[k];
+        for (uint32_t i = t; i < b.np; i += kPieceThreads) {
+            const bool is_big = i < b.big;
+            a.pieces[is_big ? b.at_big + i : b.at_q + i - b.big] =
+                make_uint4(b.s + i * b.q + (is_big ? i : b.big), is_big ? b.q + 1 : b.q, b.dest + i, 0u);
         }
     }
 }
 
-// Register caps per curve model (M::kAccBlocks blocks of 128 resident per SM), each
-// the faster of the caps measured at n = 2^20, c = 16: XYZZ at 168 registers, three
-// blocks (4 blocks: 5.75 vs 5.74 ms per accumulation; uncapped, 190 registers and two
-// blocks, slower still); Edwards at 128 registers, four blocks, with a few spills
-// (4.14 vs 4.24 ms at three blocks).
-template <class M>
-__global__ void __launch_bounds__(128, M::kAccBlocks) k_accumulate(AccArgs a) {
-    const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= (uint32_t)a.nwin * a.cpw) return;
-    accumulate_chunk<M>(a, a.w0 + (int)(id / a.cpw), id % a.cpw);
+struct AccArgs {
+    const uint32_t* items;   // sorted: stored point | sign << 31
+    const uint4* pts;
+    uint32_t npts;           // stored points
+    uint4* buckets;          // [W][Bp], four coordinates
+    uint4* parts;            // partial sums, four coordinates
+    const uint4* pieces;
+    const uint32_t* hist;    // pieces per length: their sum is the list's length
+    uint32_t cap;
+};
+
+// Pieces in the list (the same in every thread of the warp).
+__device__ __forceinline__ uint32_t piece_count(const AccArgs& a) {
+    uint32_t v = 0;
+    for (uint32_t k = threadIdx.x & 31; k <= a.cap; k += 32) v += a.hist[k];
+    return __reduce_add_sync(0xffffffffu, v);
 }
 
-// Batched MSMs: one persistent kernel drains a queue of (job, window, chunk)
-// items of all jobs. Each warp takes 32 consecutive items with one atomic.
+// Sum of one piece to its destination. What bounds it: the integer multiply pipe (7 or
+// 10 field products per point); the gather of the next point overlaps the other warps'
+// additions.
+template <class M>
+__device__ __forceinline__ void accumulate_piece(const AccArgs& a, uint32_t id) {
+    const uint4 pc = a.pieces[id];
+    const uint32_t* it = a.items + pc.x;
+    typename M::acc acc;
+    uint32_t v = it[0];
+    uint32_t idx = v & ~kSign;
+    if (idx >= a.npts) idx = 0;   // cannot happen for sorted digit output; keeps reads in bounds
+    bool inf = M::first_at(acc, a.pts, idx, (v & kSign) != 0);
+    for (uint32_t i = 1; i < pc.y; ++i) {
+        v = it[i];
+        idx = v & ~kSign;
+        if (idx >= a.npts) continue;
+        M::madd_at(acc, inf, a.pts, idx, (v & kSign) != 0);
+    }
+    uint4* d = (pc.z & kPart) ? a.parts + (size_t)(pc.z & ~kPart) * kXyzzVec : a.buckets + (size_t)pc.z * kXyzzVec;
+    M::store(d, acc);
+}
+
+// Register caps per curve model (M::kAccBlocks blocks of 128 resident per SM), each
+// the faster of the caps measured at n = 2^20, c = 16: XYZZ at 168 registers, three
+// blocks; Edwards at 128 registers, four blocks.
+template <class M>
+__global__ void __launch_bounds__(128, M::kAccBlocks) k_accumulate(AccArgs a) {
+    const uint32_t n = piece_count(a);
+    const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x;
+    if (id < n) accumulate_piece<M>(a, id);
+}
+
+// Batched MSMs: one persistent kernel drains a queue of the pieces of all jobs. Each
+// warp takes 32 consecutive places of one job's list with one atomic; a job's share of
+// the queue is its plan's bound on pieces (rounded up to 32), of which only the places
+// below its piece count hold work.
 constexpr int kMaxBatch = 128;
 struct BatchAcc {
     AccArgs job[kMaxBatch];
-    uint32_t prefix[kMaxBatch + 1];  // cumulative W * cpw over jobs
+    uint32_t prefix[kMaxBatch + 1];  // cumulative places over jobs
     int njobs;
     uint32_t* counter;
 };
@@ -1266,211 +1454,116 @@ template <class M>
 __global__ void __launch_bounds__(128, M::kAccBlocks) k_accumulate_batched(const __grid_constant__ BatchAcc b) {
     const uint32_t total = b.prefix[b.njobs];
     const int lane = threadIdx.x & 31;
+    int have = -1;       // the job whose piece count is at hand
+    uint32_t count = 0;
     for (;;) {
         uint32_t base = 0;
         if (lane == 0) base = atomicAdd(b.counter, 32u);
         base = __shfl_sync(0xffffffffu, base, 0);
         if (base >= total) break;
-        const uint32_t item = base + lane;
-        if (item < total) {
-            int lo = 0, hi = b.njobs - 1;   // last job with prefix <= item
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (b.prefix[mid] <= item) lo = mid; else hi = mid - 1;
-            }
-            const AccArgs& a = b.job[lo];
-            const uint32_t local = item - b.prefix[lo];
-            accumulate_chunk<M>(a, (int)(local / a.cpw), local % a.cpw);
+        int lo = 0, hi = b.njobs - 1;   // last job with prefix <= base
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (b.prefix[mid] <= base) lo = mid; else hi = mid - 1;
         }
-    }
-}
-
-// Partial sums of runs that cross chunk edges. When a bucket's run is expected to be
-// no longer than a chunk (items per bucket <= K), a run that continues into at most
-// kWalkHeads later chunks (every run of random scalars then) is finished by the
-// thread of its tail chunk, which adds the run's head partials in order
-// (k_merge_walk). With longer runs, serial additions on one thread would cost more
-// than the rounds below (measured at n = 2^22, c = 16: 256 items per bucket, chunks
-// of 64, 1 ms slower), so the walk is skipped and every run takes the log-depth path.
-// Longer runs are combined in log depth, so a bucket holding a large share of the
-// window (all-equal scalars, a nearly empty top window) costs O(log) serial additions,
-// not O(chunks); those kernels return at once unless the walk left such a run:
-//  * k_merge_start: for a chunk u whose first run continues an earlier chunk's
-//    run, start[u] = the chunk t0 where that run begins (its tail): the run's key
-//    first occurs at lower_bound(keys, key) in the sorted window, so t0 is that
-//    position / K (one binary search per chunk, no scan);
-//  * k_merge_round(d): for heads at offset j = u - start[u] - 1 with j % 2d == 0,
-//    head[u] += head[u + d] when u + d continues the same run; ceil(log2 cpw) rounds
-//    leave each run's sum of heads at its first head;
-//  * k_merge_long: the rounds above are launched for d < kMergeRounds only (enough for
-//    the runs of random scalars, which cross a few chunk edges); a run with more heads
-//    is finished by one block that runs the remaining rounds (d = kMergeRounds,
-//    2 kMergeRounds, ...) over that run alone between block barriers. When no run is
-//    that long the launch returns at once: one launch instead of a dozen idle rounds;
-//  * k_merge_final: bucket = tail[start] + that sum.
-constexpr uint32_t kWalkHeads = 4;
-
-template <class M>
-__global__ void k_merge_walk(AccArgs a, uint32_t H, int* __restrict__ longrun) {
-    const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= (uint32_t)a.nwin * a.cpw) return;
-    const int w = a.w0 + (int)(id / a.cpw);
-    const uint32_t t = id % a.cpw;
-    const size_t ci = (size_t)w * a.cpw + t;
-    const uint32_t key = a.tailkey[ci];
-    if (key == kNone) return;
-    typename M::acc acc;
-    M::load(acc, a.tail + ci * kXyzzVec);
-    // The run starts in chunk t (a run that began earlier would make chunk t a head);
-    // it ends where its bin ends, so it has nh = (last item) / K - t heads. Without the
-    // bin table (radix sort) the heads' flags are counted instead.
-    uint32_t nh = H + 1;
-    if (a.bin) {
-        const size_t b = (size_t)w * a.nb + key;
-        const size_t end = key + 1 < a.nb ? (size_t)a.bin[b + 1] - (size_t)w * a.n : a.n;   // within the window
-        nh = (uint32_t)((end - 1) / (size_t)a.K) - t;
-    } else {
-        for (uint32_t h = H + 1; h >= 1; --h) {
-            const uint32_t f = t + h < a.cpw ? a.headflag[ci + h] : 0u;
-            if (f == 0) nh = h - 1;      // the run ended before chunk t + h
-            if (f == 1) nh = h;          // the run ends in chunk t + h
+        const AccArgs& a = b.job[lo];
+        if (lo != have) {
+            count = piece_count(a);
+            have = lo;
         }
+        const uint32_t id = base - b.prefix[lo] + lane;
+        if (id < count) accumulate_piece<M>(a, id);
+        __syncwarp();
     }
-    if (nh > H) {                        // tail key and all, for k_merge_start .. k_merge_final
-        *longrun = 1;
-        return;
-    }
-    for (uint32_t h = 1;; ++h) {       // the heads up to the one with flag 1
-        const uint32_t f = t + h < a.cpw ? a.headflag[ci + h] : 0u;
-        if (f == 0 || h > nh) break;     // the run ended before chunk t + h
-        M::add_mem(acc, a.head + (ci + h) * kXyzzVec);
-        if (f == 1) break;               // the run ends in chunk t + h
-    }
-    M::store(a.buckets + ((size_t)w * a.Bp + (key - 1)) * kXyzzVec, acc);
-    a.tailkey[ci] = kNone;
 }
 
-// longrun: the walk's flag (null when no walk ran: every run is merged here).
-__global__ void k_merge_start(AccArgs a, const int* __restrict__ longrun, int32_t* __restrict__ start,
-                              int* __restrict__ maxspan) {
-    if (longrun && *longrun == 0) return;  // every run was finished by the walk
-    const size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (id >= (size_t)a.nwin * a.cpw) return;
-    const int w = a.w0 + (int)(id / a.cpw);
-    const uint32_t u = (uint32_t)(id % a.cpw);
-    const size_t ci = (size_t)w * a.cpw + u;
-    if (a.headflag[ci] == 0) {
-        start[ci] = -1;
-        return;
+// The block's sum of m points at `in`, four lanes per addition: group g of the block's
+// 32 groups sums in[g], in[g + 32], ... in sequence, then a tree over the groups in
+// shared memory (depth ceil(m / 32) - 1 + 5 four-lane additions). Every group of a warp
+// runs the same additions (a missing operand is the identity; idle groups of warp 0 add
+// and discard), so each __syncwarp inside them is warp-wide; a warp with no active
+// group skips a level as a whole. Thread 0 stores the sum.
+constexpr int kTreeThreads = 128;
+constexpr int kTreeGroups = kTreeThreads / 4;
+constexpr size_t kTreeWave = 152 * 3;  // blocks resident at once (3 per SM)
+
+template <class M>
+struct TreeShared {
+    uint4 pub[kTreeGroups * kXyzzVec];
+    uint4 idn[kXyzzVec];
+    fe sh[kTreeGroups][4];
+};
+
+template <class M>
+__device__ __forceinline__ void tree_init(TreeShared<M>& s) {
+    if (threadIdx.x == 0) {
+        typename M::acc e;
+        M::set_inf(e);
+        M::store(s.idn, e);
     }
-    const uint2* kv = a.kv + (size_t)w * a.n;
-    const size_t first = (size_t)u * a.K;   // u > 0 here: chunk 0 has no earlier run
-    const uint32_t key = kv[first].x;
-    size_t lo = 0, hi = first;              // first index in [0, first] with keys[i] >= key
-    while (lo < hi) {
-        const size_t mid = (lo + hi) >> 1;
-        if (kv[mid].x < key) lo = mid + 1; else hi = mid;
-    }
-    const int32_t t0 = (int32_t)(lo / (size_t)a.K);
-    start[ci] = t0;
-    atomicMax(maxspan, (int)(u - (uint32_t)t0));  // heads of this run up to u
+    __syncthreads();
 }
 
 template <class M>
-__global__ void k_merge_round(AccArgs a, const int32_t* __restrict__ start, uint32_t d,
-                              const int* __restrict__ maxspan) {
-    if (d >= (uint32_t)*maxspan) return;  // no run has heads this far apart: nothing to pair
-    const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= (uint32_t)a.nwin * a.cpw) return;
-    const int w = a.w0 + (int)(id / a.cpw);
-    const uint32_t u = id % a.cpw;
-    const size_t base = (size_t)w * a.cpw;
-    if (a.headflag[base + u] == 0) return;
-    const int32_t t0 = start[base + u];
-    if (t0 < 0) return;
-    const uint32_t j = u - (uint32_t)t0 - 1;
-    if (j % (2 * d) != 0) return;
-    const uint32_t v = u + d;
-    if (v >= a.cpw || a.headflag[base + v] == 0 || start[base + v] != t0) return;
+__device__ __forceinline__ void block_sum(TreeShared<M>& s, const uint4* __restrict__ in, uint32_t m, uint4* __restrict__ out) {
+    const int t = threadIdx.x, g = t >> 2, l = t & 3, warp = t >> 5;
     typename M::acc acc;
-    M::load(acc, a.head + (base + u) * kXyzzVec);
-    M::add_mem(acc, a.head + (base + v) * kXyzzVec);
-    M::store(a.head + (base + u) * kXyzzVec, acc);
-}
-
-constexpr uint32_t kMergeRounds = 8;   // rounds d = 1, 2, 4 launched one by one
-constexpr int kMergeLongThreads = 128;
-
-template <class M>
-__global__ void __launch_bounds__(kMergeLongThreads) k_merge_long(AccArgs a, const int32_t* __restrict__ start,
-                                                                  const int* __restrict__ maxspan) {
-    if ((uint32_t)*maxspan <= kMergeRounds) return;  // every run is complete already
-    __shared__ uint32_t first[kMergeLongThreads], span[kMergeLongThreads];
-    __shared__ uint32_t nfound;
-    const uint32_t nchunks = (uint32_t)a.nwin * a.cpw;
-    for (uint32_t tile = blockIdx.x * kMergeLongThreads; tile < nchunks; tile += gridDim.x * kMergeLongThreads) {
-        if (threadIdx.x == 0) nfound = 0;
+    if ((uint32_t)g < m)
+        M::load(acc, in + (size_t)g * kXyzzVec);
+    else
+        M::set_inf(acc);
+    for (uint32_t i0 = kTreeGroups; i0 < m; i0 += kTreeGroups) {
+        const uint32_t i = i0 + g;
+        M::add4_mem(acc, i < m ? in + (size_t)i * kXyzzVec : s.idn, s.sh[g], l);
+    }
+    // level h: groups [h, 2h) publish, groups [0, h) add them. The slots read at
+    // level h, [h, 2h), are never written at a later level (those write [h', 2h')
+    // with 2h' <= h), so one barrier per level orders every access.
+    for (int h = kTreeGroups / 2; h >= 1; h >>= 1) {
+        if ((uint32_t)h >= m) continue;   // only identities there (block-uniform)
+        if (g >= h && g < 2 * h && l == 0) M::store(s.pub + g * kXyzzVec, acc);
         __syncthreads();
-        // the first head (j = 0) of every run with more than kMergeRounds heads in this tile
-        const uint32_t id = tile + threadIdx.x;
-        if (id < nchunks) {
-            const int w = a.w0 + (int)(id / a.cpw);
-            const uint32_t u = id % a.cpw;
-            const size_t ci = (size_t)w * a.cpw + u;
-            const int32_t t0 = a.headflag[ci] != 0 ? start[ci] : -1;
-            if (t0 >= 0 && u == (uint32_t)t0 + 1) {
-                // the run's last item: the last index with this key (upper bound - 1)
-                const uint2* kv = a.kv + (size_t)w * a.n;
-                const uint32_t key = kv[(size_t)u * a.K].x;
-                size_t lo = (size_t)u * a.K, hi = a.n;
-                while (lo < hi) {
-                    const size_t mid = (lo + hi) >> 1;
-                    if (kv[mid].x <= key) lo = mid + 1; else hi = mid;
-                }
-                const uint32_t heads = (uint32_t)((lo - 1) / (size_t)a.K) - (uint32_t)t0;
-                if (heads > kMergeRounds) {
-                    const uint32_t k = atomicAdd(&nfound, 1u);
-                    first[k] = id;
-                    span[k] = heads;
-                }
-            }
+        if (warp * 8 < h) {
+            typename M::acc r = acc;
+            M::add4_mem(r, s.pub + (g + h) * kXyzzVec, s.sh[g], l);  // g + h < 32: g < h for h >= 8, g <= 7 below
+            if (g < h) acc = r;
         }
-        __syncthreads();
-        const uint32_t nf = nfound;
-        for (uint32_t r = 0; r < nf; ++r) {
-            const uint32_t f = first[r], S = span[r];
-            const int w = a.w0 + (int)(f / a.cpw);
-            const size_t h0 = (size_t)w * a.cpw + f % a.cpw;   // head j = 0 of the run
-            for (uint32_t d = kMergeRounds; d < S; d <<= 1) {
-                const uint32_t pairs = (S - d + 2 * d - 1) / (2 * d);   // j = 0, 2d, ... with j + d < S
-                for (uint32_t q = threadIdx.x; q < pairs; q += blockDim.x) {
-                    const size_t j = (size_t)q * 2 * d;
-                    typename M::acc acc;
-                    M::load(acc, a.head + (h0 + j) * kXyzzVec);
-                    M::add_mem(acc, a.head + (h0 + j + d) * kXyzzVec);
-                    M::store(a.head + (h0 + j) * kXyzzVec, acc);
-                }
-                __syncthreads();   // this level's sums are visible to the next level
-            }
-        }
-        __syncthreads();   // the list is read before the next tile overwrites it
     }
+    if (t == 0) M::store(out, acc);
 }
 
+__device__ __forceinline__ uint4* merge_dest(uint4* parts, uint4* buckets, uint32_t d) {
+    return (d & kPart) ? parts + (size_t)(d & ~kPart) * kXyzzVec : buckets + (size_t)d * kXyzzVec;
+}
+
+// One level of the merge: the tree entries by blocks, then (nsmall not null) the buckets
+// of few parts by threads.
 template <class M>
-__global__ void k_merge_final(AccArgs a, const int* __restrict__ longrun) {
-    if (longrun && *longrun == 0) return;  // every run was finished by the walk
-    const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= (uint32_t)a.nwin * a.cpw) return;
-    const int w = a.w0 + (int)(id / a.cpw);
-    const uint32_t t = id % a.cpw;
-    const size_t ci = (size_t)w * a.cpw + t;
-    const uint32_t key = a.tailkey[ci];
-    if (key == kNone) return;
-    typename M::acc acc;
-    M::load(acc, a.tail + ci * kXyzzVec);
-    if (t + 1 < a.cpw && a.headflag[ci + 1] != 0) M::add_mem(acc, a.head + (ci + 1) * kXyzzVec);
-    M::store(a.buckets + ((size_t)w * a.Bp + (key - 1)) * kXyzzVec, acc);
+__global__ void __launch_bounds__(kTreeThreads) k_merge_parts(uint4* parts, uint4* buckets, const uint4* __restrict__ tree,
+                                                              const uint32_t* __restrict__ ntree,
+                                                              const uint4* __restrict__ small,
+                                                              const uint32_t* __restrict__ nsmall) {
+    __shared__ TreeShared<M> s;
+    const uint32_t nt = *ntree;
+    if (blockIdx.x < nt) {
+        tree_init(s);
+        for (uint32_t e = blockIdx.x; e < nt; e += gridDim.x) {
+            const uint4 x = tree[e];
+            block_sum(s, parts + (size_t)x.x * kXyzzVec, x.y, merge_dest(parts, buckets, x.z));
+            __syncthreads();   // the published points are read before the next entry's
+        }
+    }
+    if (!nsmall) return;
+    const uint32_t ns = *nsmall;
+    // from the last block down: the first ones have the tree entries
+    for (uint32_t i = (gridDim.x - 1 - blockIdx.x) * kTreeThreads + threadIdx.x; i < ns; i += gridDim.x * kTreeThreads) {
+        const uint4 x = small[i];
+        const uint4* p = parts + (size_t)x.x * kXyzzVec;
+        typename M::acc acc;
+        M::load(acc, p);
+        for (uint32_t k = 1; k < x.y; ++k) M::add_mem(acc, p + (size_t)k * kXyzzVec);
+        M::store(buckets + (size_t)x.z * kXyzzVec, acc);
+    }
 }
 
 // ---------------------------------------------------------------- stage 6
@@ -1524,58 +1617,20 @@ __global__ void k_bitsums(const uint4* __restrict__ Y, const uint4* __restrict__
 }
 
 // Block (s, b) sums in[s][F 32 b .. F 32 (b + 1) - 1] (within the segment's m points)
-// into out[s][b] with four lanes per addition: group j of the block's 32 groups sums
-// in[F 32 b + j + 32 f] for f < F in sequence, then a tree over the groups in shared
-// memory (depth F - 1 + 5 four-lane additions; a segment of m points needs
-// log_(32 F) m launches; F is chosen so that a launch fills about one wave of
-// blocks). Every group of a warp runs the same additions (a missing operand is the
-// identity; idle groups of warp 0 add and discard), so each __syncwarp inside them
-// is warp-wide; a warp with no active group skips a level as a whole.
-constexpr int kTreeThreads = 128;
-constexpr int kTreeGroups = kTreeThreads / 4;
-constexpr size_t kTreeWave = 152 * 3;  // blocks resident at once (3 per SM)
-
+// into out[s][b]; a segment of m points needs log_(32 F) m launches. F is chosen so that
+// a launch fills about one wave of blocks.
 template <class M>
 __global__ void __launch_bounds__(kTreeThreads) k_sum_tree(const uint4* __restrict__ in, size_t nseg, uint32_t m,
                                                           uint32_t F, uint4* __restrict__ out) {
-    __shared__ uint4 pub[kTreeGroups * kXyzzVec];
-    __shared__ uint4 idn[kXyzzVec];
-    __shared__ fe sh[kTreeGroups][4];
+    __shared__ TreeShared<M> s;
     const uint32_t per = kTreeGroups * F;
     const uint32_t nb = (m + per - 1) / per;
     const size_t seg = blockIdx.x / nb;
     const uint32_t b = blockIdx.x % nb;
     if (seg >= nseg) return;  // whole block
-    const int t = threadIdx.x, g = t >> 2, l = t & 3, warp = t >> 5;
-    if (t == 0) {
-        typename M::acc e;
-        M::set_inf(e);
-        M::store(idn, e);
-    }
-    __syncthreads();
-    const uint32_t i0 = b * per + g;
-    typename M::acc acc;
-    if (i0 < m)
-        M::load(acc, in + (seg * m + i0) * kXyzzVec);
-    else
-        M::set_inf(acc);
-    for (uint32_t f = 1; f < F; ++f) {
-        const uint32_t i = i0 + f * kTreeGroups;
-        M::add4_mem(acc, i < m ? in + (seg * m + i) * kXyzzVec : idn, sh[g], l);
-    }
-    // level h: groups [h, 2h) publish, groups [0, h) add them. The slots read at
-    // level h, [h, 2h), are never written at a later level (those write [h', 2h')
-    // with 2h' <= h), so one barrier per level orders every access.
-    for (int h = kTreeGroups / 2; h >= 1; h >>= 1) {
-        if (g >= h && g < 2 * h && l == 0) M::store(pub + g * kXyzzVec, acc);
-        __syncthreads();
-        if (warp * 8 < h) {
-            typename M::acc r = acc;
-            M::add4_mem(r, pub + (g + h) * kXyzzVec, sh[g], l);  // g + h < 32: g < h for h >= 8, g <= 7 below
-            if (g < h) acc = r;
-        }
-    }
-    if (t == 0) M::store(out + (seg * nb + b) * kXyzzVec, acc);
+    tree_init(s);
+    const uint32_t left = m - b * per;
+    block_sum(s, in + (seg * m + (size_t)b * per) * kXyzzVec, left < per ? left : per, out + (seg * nb + b) * kXyzzVec);
 }
 
 // ---------------------------------------------------------------- stage 7
@@ -1652,21 +1707,22 @@ struct Plan {
     uint32_t B, Bp;
     int passes, rb;  // radix-sort passes of rb-bit digits
     size_t tiles;
-    int K;
-    uint32_t cpw;   // chunks per window
+    int K;          // longest piece of a bucket's run
+    uint32_t small_parts;   // parts that one thread puts together
+    size_t max_pieces, max_parts, max_small, max_tree[3];   // per group: bounds over any digits
     int gw;         // windows per group
     int ngroups;
     uint32_t L, G, Q;
     int logG, log2L;
-    size_t off_status, off_points, off_keys0, off_vals0, off_keys1, off_vals1, off_kv, off_rank, off_hist, off_dtot;
+    size_t off_status, off_ctrl, ctrl_bytes;   // status words, then the groups' counters: cleared together
+    size_t off_points, off_keys0, off_vals0, off_keys1, off_vals1, off_rank, off_hist, off_dtot;
     int counting;                      // counting sort (else LSD radix sort)
     size_t nbins, off_bins, off_bsum;  // counting sort: bins (window, key) and scan tile totals
     uint32_t ttiles, tT;               // counting sort in shared-memory tiles: tiles per window, items per
                                        // tile (ttiles = 0: global counters)
     size_t off_tcnt;                   // per-tile counts and prefixes [W][ttiles][Bp + 1]
-    uint32_t walk;                     // heads a run's tail thread adds itself (0: no walk)
-    size_t off_buckets, off_head, off_tail, off_headflag, off_tailkey, off_Y, off_V, off_P0, off_P1;
-    size_t off_S, off_start, total;
+    size_t off_buckets, off_parts, off_pieces, off_small, off_tree[3], off_Y, off_V, off_P0, off_P1;
+    size_t off_S, total;
 };
 
 constexpr uint64_t kReduceThreads = 32768;
@@ -1707,9 +1763,6 @@ int default_c(size_t n, int sgn, uint32_t flags) {
 }
 
 constexpr int kMaxGroups = 8;
-// status words: the call's status, then per window group the longest run's head count
-// (k_merge_start) and whether a run outgrew the walk (k_merge_walk)
-constexpr int kStatusWords = 1 + 2 * kMaxGroups;
 
 // allow_groups = false: one window group (batched calls overlap whole jobs instead).
 bool make_plan(size_t n, const msm_opts* o, Plan* p, bool allow_groups = true) {
@@ -1788,22 +1841,40 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool allow_groups = true) {
     }
     p->gw = (p->W + groups - 1) / groups;
     p->ngroups = (p->W + p->gw - 1) / p->gw;
-    // Chunks of K <= 64 items, one per thread, sized so that the chunks of one
-    // accumulation launch (one window group) fill whole waves of resident threads
-    // (152 SMs x kAccBlocks blocks of 128 on a GB300): m waves of K items rather than
-    // a last, partly idle wave.
+    // Pieces of at most K items, one thread each (stage 4): K = the mean run plus four
+    // standard deviations, so that with at least a wave of buckets only unusually long
+    // runs are cut (random digits leave hardly any); up to a third of a resident thread's
+    // share of all items, so that a piece never outlasts the rest of the work, and up
+    // to two shares, so that every resident thread (152 SMs x kAccBlocks blocks of 128 on
+    // a GB300) has work where buckets are few.
     const size_t kWave = (size_t)152 * 128 * (p->edw ? ModelEdwards::kAccBlocks : ModelXyzz::kAccBlocks);
     const size_t total = (size_t)p->gw * items;
-    size_t waves = (total + 64 * kWave - 1) / (64 * kWave);
-    if (waves < 1) waves = 1;
-    size_t K = (total + waves * kWave - 1) / (waves * kWave);
+    const size_t mean = (items + p->B - 1) / p->B;      // items per bucket of a full window
+    size_t K = mean + 8;
+    while ((K - mean) * (K - mean) < 16 * mean) ++K;    // mean + 4 sqrt(mean)
+    const size_t share = (total + kWave - 1) / kWave;
+    if (K < share / 3) K = share / 3;
+    if (K > 2 * share + 4) K = 2 * share + 4;
     if (K < 2) K = 2;
-    if (K > 64) K = 64;
+    if (K > kMaxPiece) K = kMaxPiece;
     if (tk > 0) K = (size_t)tk;        // measured choice (2..256)
     p->K = (int)K;
-    p->cpw = (uint32_t)((items + K - 1) / K);
-    p->walk = (items + p->Bp - 1) / p->Bp <= K ? kWalkHeads : 0u;   // runs about a chunk long at most
-    if (p->cpw == 0) p->cpw = 1;
+    {
+        // sum over buckets of ceil(m / K): at most one piece more than m / K per bucket in
+        // use; a bucket with parts has more than K items
+        const size_t nbk = (size_t)p->gw * p->Bp, used = nbk < total ? nbk : total;
+        const size_t cut = total / (K + 1) < nbk ? total / (K + 1) : nbk;
+        p->max_pieces = total / K + used;
+        const size_t multi = total / K + cut;
+        p->max_parts = multi + multi / 2;               // and the tree levels' sums
+        p->max_small = cut;
+        // With many buckets the threads' sequential sums fill the GPU; few buckets' parts
+        // go to blocks (816 buckets of 8 parts, XYZZ: 195 us by blocks, 280 us by threads).
+        p->small_parts = nbk >= 2048 ? 8 : 2;
+        p->max_tree[0] = multi / (p->small_parts + 1) + 1;
+        p->max_tree[1] = p->max_tree[2] = multi / kTreeParts + 1;
+        if (p->max_parts >= kPart || p->max_pieces >= (1ull << 32)) return false;
+    }
     // bucket reduction geometry: segments of L buckets, the longest L that still
     // leaves kReduceThreads level-1 threads over all windows (longer segments mean
     // fewer segment sums for the bit-sum stage, but fewer threads for the running sums)
@@ -1825,18 +1896,17 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool allow_groups = true) {
         return o2;
     };
     const size_t XY = kXyzzBytes;
-    const size_t chunks = (size_t)p->W * p->cpw;
     p->off_status = take(256);
+    p->off_ctrl = take((size_t)p->ngroups * kCtrlWords * 4);
+    p->ctrl_bytes = p->off_ctrl + (size_t)p->ngroups * kCtrlWords * 4 - p->off_status;
     p->off_points = take(o->flags & MSM377_POINTS_PREPARED ? 0 : np * 16 * (size_t)p->stored_vec);
-    p->off_keys0 = take((size_t)p->W * items * 4);
-    p->off_vals0 = take((size_t)p->W * items * 4);
-    // the sort's ping-pong buffers (radix passes before the last); the last pass, or
-    // the counting scatter, writes (key, value) pairs to kv
-    const bool pingpong = !p->counting && p->passes > 1;
-    p->off_keys1 = take(pingpong ? (size_t)p->W * items * 4 : 0);
-    p->off_vals1 = take(pingpong ? (size_t)p->W * items * 4 : 0);
-    p->off_kv = take((size_t)p->W * items * 8);
-    p->off_rank = take(p->counting ? (size_t)p->W * items * 4 : 0);  // counting sort: rank within the bin
+    const size_t all = (size_t)p->W * items;
+    p->off_keys0 = take(all * 4);
+    p->off_vals0 = take(all * 4);
+    // the radix sort's ping-pong buffers
+    p->off_keys1 = take(p->counting ? 0 : all * 4);
+    p->off_vals1 = take(p->counting ? 0 : all * 4);
+    p->off_rank = take(p->counting ? all * 4 : 0);  // counting sort: rank within the bin
     p->off_hist = take((size_t)p->W * (1u << p->rb) * (p->tiles ? p->tiles : 1) * 4);
     p->off_dtot = take((size_t)p->W * (1u << p->rb) * 4);
     p->nbins = (size_t)p->W * (p->Bp + 1);  // keys 0 .. Bp of every window
@@ -1844,11 +1914,10 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool allow_groups = true) {
     p->off_bsum = take(((p->nbins + kScanTile - 1) / kScanTile) * 4);
     p->off_tcnt = take((size_t)p->W * p->ttiles * (p->Bp + 1) * 4);
     p->off_buckets = take((size_t)p->W * p->Bp * XY);
-    p->off_head = take(chunks * XY);
-    p->off_tail = take(chunks * XY);
-    p->off_headflag = take(chunks * 4);
-    p->off_tailkey = take(chunks * 4);
-    p->off_start = take(chunks * 4);
+    p->off_parts = take(p->ngroups * p->max_parts * XY);
+    p->off_pieces = take(p->ngroups * p->max_pieces * 16);
+    p->off_small = take(p->ngroups * p->max_small * 16);
+    for (int k = 0; k < 3; ++k) p->off_tree[k] = take(p->ngroups * p->max_tree[k] * 16);
     p->off_Y = take((size_t)p->ngroups * p->gw * p->G * XY);    // per group
     p->off_V = take((size_t)p->ngroups * p->gw * p->G * XY);
     const size_t zs = (size_t)p->gw * (p->logG + 1) * p->Q;
@@ -2023,16 +2092,53 @@ extern "C" int msm_points_precompute(const uint32_t* points_std, size_t n, uint3
 
 namespace {
 
-// Phase 1-3 of one MSM on stream s: status reset, preparation, digits, sort,
-// bucket reset. Fills `a` with the job's accumulation arguments.
-// reset_status = false: the caller has cleared the status word and the merge
-// counter already (msm_g1_host validates point chunks on a helper stream first).
+// Phase 1-3 of one MSM on stream s: counters reset, preparation, digits, sort, and the
+// pieces of every window group. Fills `job` with what the accumulations and tails need.
+// reset_status = false: the caller has cleared the status word and the counters
+// already (msm_g1_host validates point chunks on a helper stream first).
+struct Job {
+    const uint4* pts;
+    const uint32_t* items;
+};
+
+PieceArgs piece_args(const Plan& p, void* workspace, int g) {
+    PieceArgs a;
+    a.start = at<uint32_t>(workspace, p.off_bins);
+    a.nb = p.Bp + 1;
+    a.Bp = p.Bp;
+    a.w0 = g * p.gw;
+    a.nwin = p.W - a.w0 < p.gw ? p.W - a.w0 : p.gw;
+    a.total = (uint32_t)((size_t)(a.w0 + a.nwin) * p.items);
+    a.cap = (uint32_t)p.K;
+    a.small_parts = p.small_parts;
+    a.ctrl = at<uint32_t>(workspace, p.off_ctrl) + (size_t)g * kCtrlWords;
+    a.pieces = at<uint4>(workspace, p.off_pieces) + (size_t)g * p.max_pieces;
+    a.small = at<uint4>(workspace, p.off_small) + (size_t)g * p.max_small;
+    for (int k = 0; k < 3; ++k) a.tree[k] = at<uint4>(workspace, p.off_tree[k]) + (size_t)g * p.max_tree[k];
+    a.buckets = at<uint4>(workspace, p.off_buckets);
+    return a;
+}
+
+AccArgs acc_args(const Plan& p, const Job& job, void* workspace, int g) {
+    const PieceArgs pa = piece_args(p, workspace, g);
+    AccArgs a;
+    a.items = job.items;
+    a.pts = job.pts;
+    a.npts = (uint32_t)p.items;   // stored rows: np, or Wd np with precomputed copies
+    a.buckets = pa.buckets;
+    a.parts = at<uint4>(workspace, p.off_parts) + (size_t)g * p.max_parts * kXyzzVec;
+    a.pieces = pa.pieces;
+    a.hist = pa.ctrl + kHist;
+    a.cap = pa.cap;
+    return a;
+}
+
 int enqueue_head(const Plan& p, const uint32_t* points, const uint32_t* scalars, void* workspace,
-                 const msm_opts* opts, cudaStream_t s, AccArgs* a_out, bool reset_status = true) {
+                 const msm_opts* opts, cudaStream_t s, Job* job, bool reset_status = true) {
     const size_t n = p.n;
     int* status = at<int>(workspace, p.off_status);
     if (reset_status)
-        MSM_CUDA_TRY(cudaMemsetAsync(status, 0, kStatusWords * sizeof(int), s));  // status, longest runs
+        MSM_CUDA_TRY(cudaMemsetAsync(status, 0, p.ctrl_bytes, s));
     const uint4* pts = reinterpret_cast<const uint4*>(points);
     if ((opts->flags & MSM377_VALIDATE) && !(opts->flags & MSM377_POINTS_PREPARED)) {
         const int r = launch_validate(points, n, (opts->flags & (MSM377_EDWARDS | MSM377_GLV)) != 0, status, s);
@@ -2046,16 +2152,16 @@ int enqueue_head(const Plan& p, const uint32_t* points, const uint32_t* scalars,
     const size_t np = p.items;  // items per pipeline window
     uint32_t* keys[2] = {at<uint32_t>(workspace, p.off_keys0), at<uint32_t>(workspace, p.off_keys1)};
     uint32_t* vals[2] = {at<uint32_t>(workspace, p.off_vals0), at<uint32_t>(workspace, p.off_vals1)};
-    uint2* kv = at<uint2>(workspace, p.off_kv);
     k_digits<<<grid_for(n, 256), 256, 0, s>>>(reinterpret_cast<const uint4*>(scalars), n, p.c, p.Wd,
-                                              p.sgn, p.user_bits, p.glv, p.pre, keys[0], vals[0], status);
+                                              p.sgn, p.user_bits, p.glv, keys[0], status);
     note_launches(1);
     int cur = 0;
+    const int pre_w = p.pre ? p.Wd : 0;
+    const uint32_t nb = p.Bp + 1;
+    uint32_t* bins = at<uint32_t>(workspace, p.off_bins);
     if (p.counting) {
         // counting sort: count, scan, scatter (window-major bins, window w at w np)
         const size_t total = (size_t)p.W * np;
-        const uint32_t nb = p.Bp + 1;
-        uint32_t* bins = at<uint32_t>(workspace, p.off_bins);
         uint32_t* bsum = at<uint32_t>(workspace, p.off_bsum);
         uint32_t* rank = at<uint32_t>(workspace, p.off_rank);
         const size_t ntiles = (p.nbins + kScanTile - 1) / kScanTile;
@@ -2078,9 +2184,9 @@ int enqueue_head(const Plan& p, const uint32_t* points, const uint32_t* scalars,
         k_scan_add<<<grid_for(p.nbins, 256), 256, 0, s>>>(bins, p.nbins, bsum);
         if (p.ttiles) {
             k_tile_offsets<<<grid_for(p.nbins, 256), 256, 0, s>>>(tcnt, nb, p.ttiles, (uint32_t)p.W, bins);
-            k_tile_scatter<<<gw, 256, 0, s>>>(keys[0], vals[0], rank, kv, total, np, nb, p.tT, p.ttiles, tcnt);
+            k_tile_scatter<<<gw, 256, 0, s>>>(keys[0], rank, vals[0], total, np, nb, p.tT, p.ttiles, tcnt, p.np, pre_w);
         } else {
-            k_bin_scatter<<<gw, 256, 0, s>>>(keys[0], vals[0], rank, kv, total, np, nb, bins);
+            k_bin_scatter<<<gw, 256, 0, s>>>(keys[0], rank, vals[0], total, np, nb, bins, p.np, pre_w);
         }
         note_launches(p.ttiles ? 7 : 5);
     } else {
@@ -2092,39 +2198,30 @@ int enqueue_head(const Plan& p, const uint32_t* points, const uint32_t* scalars,
             k_sort_hist<8><<<g, kSortThreads, 0, s>>>(keys[cur], np, shift, p.tiles, hist);
             k_sort_scan_tiles<8><<<dim3(1u << 8, p.W), kSortThreads, 0, s>>>(hist, p.tiles, dtot);
             k_sort_scan_digits<8><<<p.W, kSortThreads, 0, s>>>(dtot);
-            uint2* last = pass == p.passes - 1 ? kv : nullptr;
-            k_sort_scatter<8><<<g, kSortThreads, 0, s>>>(keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], last,
-                                                         np, shift, p.tiles, hist, dtot);
+            k_sort_scatter<8><<<g, kSortThreads, 0, s>>>(keys[cur], pass ? vals[cur] : nullptr, keys[cur ^ 1],
+                                                         vals[cur ^ 1], np, shift, p.tiles, hist, dtot, p.np, pre_w);
             note_launches(4);
             cur ^= 1;
         }
+        k_run_starts<<<dim3(grid_for(np, 256), (unsigned)p.W), 256, 0, s>>>(keys[cur], np, nb, bins);
+        note_launches(1);
     }
-    uint4* buckets = at<uint4>(workspace, p.off_buckets);
-    MSM_CUDA_TRY(cudaMemsetAsync(buckets, 0, (size_t)p.W * p.Bp * kXyzzBytes, s));
-    AccArgs& a = *a_out;
-    a.kv = kv;
-    a.pts = pts;
-    a.buckets = buckets;
-    a.head = at<uint4>(workspace, p.off_head);
-    a.tail = at<uint4>(workspace, p.off_tail);
-    a.headflag = at<uint32_t>(workspace, p.off_headflag);
-    a.tailkey = at<uint32_t>(workspace, p.off_tailkey);
-    a.n = np;
-    a.cpw = p.cpw;
-    a.Bp = p.Bp;
-    a.K = p.K;
-    a.w0 = 0;
-    a.nwin = p.W;
-    a.bin = p.counting ? at<uint32_t>(workspace, p.off_bins) : nullptr;
-    a.nb = p.Bp + 1;
+    job->pts = pts;
+    job->items = vals[cur];
+    for (int g = 0; g < p.ngroups; ++g) {
+        const PieceArgs a = piece_args(p, workspace, g);
+        const unsigned grid = grid_for((size_t)a.nwin * nb, kPieceThreads);
+        k_piece_count<<<grid, kPieceThreads, 0, s>>>(a);
+        k_piece_emit<<<grid, kPieceThreads, 0, s>>>(a);
+        note_launches(2);
+    }
     return check_launch("msm head");
 }
 
-// Phase 5-6 and the per-window sums of stage 7 for the windows of one group
-// (a.w0 .. a.w0 + a.nwin - 1) on stream s: partial merges, bucket reduction, and
-// S_w for each window, in group g's buffers.
+// Phase 5-6 and the per-window sums of stage 7 for the windows of group g on stream s:
+// partial merges, bucket reduction, and S_w for each window, in the group's buffers.
 template <class M>
-int enqueue_group_tail_m(const Plan& p, const AccArgs& a, int g, void* workspace, cudaStream_t s) {
+int enqueue_group_tail_m(const Plan& p, const AccArgs& acc, int g, void* workspace, cudaStream_t s) {
     const size_t yv = (size_t)p.gw * p.G * kXyzzVec;
     const size_t zs = (size_t)p.gw * (p.logG + 1) * p.Q * kXyzzVec;
     uint4* Y = at<uint4>(workspace, p.off_Y) + (size_t)g * yv;
@@ -2132,33 +2229,17 @@ int enqueue_group_tail_m(const Plan& p, const AccArgs& a, int g, void* workspace
     uint4* P0 = at<uint4>(workspace, p.off_P0) + (size_t)g * zs;
     uint4* P1 = at<uint4>(workspace, p.off_P1) + (size_t)g * zs;
     int* S = at<int>(workspace, p.off_S);
-    const size_t nchunks = (size_t)a.nwin * p.cpw;
-    // 5. merge partial sums of runs crossing chunk edges (log depth)
-    int32_t* start = at<int32_t>(workspace, p.off_start);
-    int* maxspan = at<int>(workspace, p.off_status) + 1 + g;
-    // the walk's flag, or null without a walk (a one-byte memset in its place made 64
-    // graph-captured batched MSMs 37 -> 52 ms on GB300)
-    int* longrun = p.walk ? at<int>(workspace, p.off_status) + 1 + kMaxGroups + g : nullptr;
-    if (p.walk) {
-        k_merge_walk<M><<<grid_for(nchunks, 128), 128, 0, s>>>(a, p.walk, longrun);
+    const PieceArgs a = piece_args(p, workspace, g);
+    // 5. the parts of buckets cut into pieces, as many tree levels as a bucket can need
+    const size_t most = (p.items + p.K - 1) / p.K;   // pieces of one bucket
+    size_t per = 1;
+    for (int lv = 0; lv < 3 && most > per; ++lv, per *= kTreeParts) {
+        const size_t want = p.max_tree[lv] + (lv == 0 ? (p.max_small + kTreeThreads - 1) / kTreeThreads : 0);
+        k_merge_parts<M><<<(unsigned)(want < kTreeWave ? want : kTreeWave), kTreeThreads, 0, s>>>(
+            acc.parts, acc.buckets, a.tree[lv], a.ctrl + kNTree + lv, lv == 0 ? a.small : nullptr,
+            lv == 0 ? a.ctrl + kNSmall : nullptr);
         note_launches(1);
     }
-    k_merge_start<<<grid_for(nchunks, 128), 128, 0, s>>>(a, longrun, start, maxspan);
-    note_launches(1);
-    for (uint32_t d = 1; d < p.cpw && d < kMergeRounds; d <<= 1) {
-        k_merge_round<M><<<grid_for(nchunks, 128), 128, 0, s>>>(a, start, d, maxspan);
-        note_launches(1);
-    }
-    if (p.cpw > kMergeRounds) {
-        int dev = 0, sms = 152;
-        MSM_CUDA_TRY(cudaGetDevice(&dev));
-        MSM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const size_t want = (nchunks + kMergeLongThreads - 1) / kMergeLongThreads, cap = (size_t)sms * 4;
-        k_merge_long<M><<<(unsigned)(want < cap ? want : cap), kMergeLongThreads, 0, s>>>(a, start, maxspan);
-        note_launches(1);
-    }
-    k_merge_final<M><<<grid_for(nchunks, 128), 128, 0, s>>>(a, longrun);
-    note_launches(1);
     // 6. bucket reduction of the group's windows
     const size_t WG = (size_t)a.nwin * p.G;
     k_reduce_segments<M><<<grid_for(WG, 128), 128, 0, s>>>(a.buckets, p.Bp, p.L, a.w0, a.nwin, p.G, Y, V);
@@ -2208,9 +2289,9 @@ int enqueue_tail(const Plan& p, const AccArgs& a, void* workspace, uint32_t* out
     return enqueue_chain(p, workspace, out, s);
 }
 
-// Accumulation of the windows a.w0 .. a.w0 + a.nwin - 1.
+// Accumulation of one window group.
 int enqueue_accumulate(const Plan& p, const AccArgs& a, cudaStream_t s) {
-    const unsigned grid = grid_for((size_t)a.nwin * p.cpw, 128);
+    const unsigned grid = grid_for(p.max_pieces, 128);
     if (p.edw)
         k_accumulate<ModelEdwards><<<grid, 128, 0, s>>>(a);
     else
@@ -2262,32 +2343,22 @@ const Overlap* overlap_for(cudaStream_t s) {
 // group's accumulation), then the window chain on s. Without a helper (ov null, or
 // one group) everything runs in order on s. prof: stage marks after the last
 // accumulation and after the chain.
-int enqueue_body(const Plan& p, const AccArgs& a, void* workspace, uint32_t* out, cudaStream_t s, const Overlap* ov,
+int enqueue_body(const Plan& p, const Job& job, void* workspace, uint32_t* out, cudaStream_t s, const Overlap* ov,
                  bool prof) {
     int r;
     if (p.ngroups <= 1 || !ov) {
-        for (int g = 0; g < p.ngroups; ++g) {
-            AccArgs ag = a;
-            ag.w0 = g * p.gw;
-            ag.nwin = (p.W - ag.w0) < p.gw ? (p.W - ag.w0) : p.gw;
-            if ((r = enqueue_accumulate(p, ag, s))) return r;
-        }
+        for (int g = 0; g < p.ngroups; ++g)
+            if ((r = enqueue_accumulate(p, acc_args(p, job, workspace, g), s))) return r;
         if (prof) profile_mark(s);
-        for (int g = 0; g < p.ngroups; ++g) {
-            AccArgs ag = a;
-            ag.w0 = g * p.gw;
-            ag.nwin = (p.W - ag.w0) < p.gw ? (p.W - ag.w0) : p.gw;
-            if ((r = enqueue_group_tail(p, ag, g, workspace, s))) return r;
-        }
+        for (int g = 0; g < p.ngroups; ++g)
+            if ((r = enqueue_group_tail(p, acc_args(p, job, workspace, g), g, workspace, s))) return r;
     } else {
         for (int g = 0; g < p.ngroups; ++g) {
-            AccArgs ag = a;
-            ag.w0 = g * p.gw;
-            ag.nwin = (p.W - ag.w0) < p.gw ? (p.W - ag.w0) : p.gw;
-            if ((r = enqueue_accumulate(p, ag, s))) return r;
+            const AccArgs a = acc_args(p, job, workspace, g);
+            if ((r = enqueue_accumulate(p, a, s))) return r;
             MSM_CUDA_TRY(cudaEventRecord(ov->ev[g], s));
             MSM_CUDA_TRY(cudaStreamWaitEvent(ov->hi, ov->ev[g], 0));
-            if ((r = enqueue_group_tail(p, ag, g, workspace, ov->hi))) return r;
+            if ((r = enqueue_group_tail(p, a, g, workspace, ov->hi))) return r;
         }
         if (prof) profile_mark(s);
         MSM_CUDA_TRY(cudaEventRecord(ov->ev[kMaxGroups], ov->hi));
@@ -2386,7 +2457,7 @@ int msm_g1_run(const uint32_t* points, const uint32_t* scalars, size_t n, uint32
     }
     if (!points || !scalars || !aligned(points, 16) || !aligned(scalars, 16))
         return set_error(MSM377_EINVAL, "msm_g1: points/scalars NULL or not 16-byte aligned");
-    AccArgs a;
+    Job job;
     // Standard-form points: their preparation (and validation) runs on the caller
     // stream's high-priority helper while the digits and the sort, which need only
     // the scalars, run on s; the accumulation waits for both.
@@ -2395,7 +2466,7 @@ int msm_g1_run(const uint32_t* points, const uint32_t* scalars, size_t n, uint32
     int r;
     if (split && ov) {
         int* status = at<int>(workspace, p.off_status);
-        MSM_CUDA_TRY(cudaMemsetAsync(status, 0, kStatusWords * sizeof(int), s));
+        MSM_CUDA_TRY(cudaMemsetAsync(status, 0, p.ctrl_bytes, s));
         MSM_CUDA_TRY(cudaEventRecord(ov->ev[0], s));
         MSM_CUDA_TRY(cudaStreamWaitEvent(ov->hi, ov->ev[0], 0));
         if (opts->flags & MSM377_VALIDATE) {
@@ -2407,15 +2478,15 @@ int msm_g1_run(const uint32_t* points, const uint32_t* scalars, size_t n, uint32
         MSM_CUDA_TRY(cudaEventRecord(ov->ev[1], ov->hi));
         msm_opts op = *opts;
         op.flags |= MSM377_POINTS_PREPARED;  // the plan keeps the prepared region in the workspace
-        r = enqueue_head(p, reinterpret_cast<const uint32_t*>(prep), scalars, workspace, &op, s, &a, false);
+        r = enqueue_head(p, reinterpret_cast<const uint32_t*>(prep), scalars, workspace, &op, s, &job, false);
         if (r) return r;
         MSM_CUDA_TRY(cudaStreamWaitEvent(s, ov->ev[1], 0));
     } else {
-        r = enqueue_head(p, points, scalars, workspace, opts, s, &a);
+        r = enqueue_head(p, points, scalars, workspace, opts, s, &job);
         if (r) return r;
     }
     if (prof) profile_mark(s);
-    return enqueue_body(p, a, workspace, out, s, p.ngroups > 1 ? ov : nullptr, prof);
+    return enqueue_body(p, job, workspace, out, s, p.ngroups > 1 ? ov : nullptr, prof);
 }
 
 }  // namespace msm377
@@ -2497,9 +2568,11 @@ extern "C" int msm_g1_batched(const msm_job* jobs, size_t njobs, void* workspace
             MSM_CUDA_TRY(cudaMemsetAsync(jobs[i].out, 0, 24 * sizeof(uint32_t), si));
             continue;
         }
-        r = enqueue_head(plans[i], jobs[i].points, jobs[i].scalars, ws[i], opts, si, &b.job[b.njobs]);
+        Job job;
+        r = enqueue_head(plans[i], jobs[i].points, jobs[i].scalars, ws[i], opts, si, &job);
         if (r) return r;
-        b.prefix[b.njobs + 1] = b.prefix[b.njobs] + (uint32_t)(plans[i].W * plans[i].cpw);
+        b.job[b.njobs] = acc_args(plans[i], job, ws[i], 0);
+        b.prefix[b.njobs + 1] = b.prefix[b.njobs] + (uint32_t)((plans[i].max_pieces + 31) / 32 * 32);
         ++b.njobs;
     }
     r = join_into(aux, s, nst);
@@ -2587,7 +2660,7 @@ extern "C" int msm_g1_host(const uint32_t* points_host, const uint32_t* scalars_
     int r = device_aux(&aux);
     if (r) return r;
     cudaStream_t sc = aux->st[0];
-    MSM_CUDA_TRY(cudaMemsetAsync(at<int>(workspace, p.off_status), 0, kStatusWords * sizeof(int), s));  // before the fork
+    MSM_CUDA_TRY(cudaMemsetAsync(at<int>(workspace, p.off_status), 0, p.ctrl_bytes, s));  // before the fork
     r = fork_from(aux, s, 1 + kHostChunks);
     if (r) return r;
     uint4* prep = at<uint4>(workspace, p.off_points);
@@ -2609,12 +2682,12 @@ extern "C" int msm_g1_host(const uint32_t* points_host, const uint32_t* scalars_
     MSM_CUDA_TRY(cudaMemcpyAsync(d_sc, scalars_host, n * 32, cudaMemcpyHostToDevice, s));
     msm_opts op = o;
     op.flags |= MSM377_POINTS_PREPARED;  // the plan above keeps the prepared region in the workspace
-    AccArgs acc;
-    r = enqueue_head(p, reinterpret_cast<const uint32_t*>(prep), d_sc, workspace, &op, s, &acc, false);
+    Job job;
+    r = enqueue_head(p, reinterpret_cast<const uint32_t*>(prep), d_sc, workspace, &op, s, &job, false);
     if (r) return r;
     r = join_into(aux, s, 1 + kHostChunks);
     if (r) return r;
-    r = enqueue_body(p, acc, workspace, d_out, s, p.ngroups > 1 ? overlap_for(s) : nullptr, false);
+    r = enqueue_body(p, job, workspace, d_out, s, p.ngroups > 1 ? overlap_for(s) : nullptr, false);
     if (r) return r;
     MSM_CUDA_TRY(cudaMemcpyAsync(out_host, d_out, 24 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     return msm_g1_status(workspace, &o);
