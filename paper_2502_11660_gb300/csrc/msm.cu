@@ -142,6 +142,7 @@ struct ModelXyzz {
         if (negate) ec::neg(Q);
         ec::madd(P, inf, Q);
     }
+    static __device__ __forceinline__ bool empty(const uint4*) { return false; }  // ZZ = 0 is the identity
     static __device__ __forceinline__ void add_mem(acc& P, const uint4* q) { ec::add_q(P, MemQ{q}); }
     static __device__ __forceinline__ void add(acc& P, const acc& Q) { ec::add(P, Q); }
     static __device__ __forceinline__ void add4_mem(acc& P, const uint4* q, fe* sh, int l) {
@@ -186,11 +187,13 @@ struct ModelEdwards {
         load_stored(Q, pts, idx, negate);
         ed::madd(P, Q);
     }
-    static __device__ __forceinline__ void add_mem(acc& P, const uint4* q) {
+    static __device__ __forceinline__ bool empty(const uint4* q) {
         fe z;
         load_fe(z, q + 6);
-        if (fq::is_zero_raw(z)) return;  // empty bucket
-        ed::add_q(P, MemQE{q});
+        return fq::is_zero_raw(z);
+    }
+    static __device__ __forceinline__ void add_mem(acc& P, const uint4* q) {
+        if (!empty(q)) ed::add_q(P, MemQE{q});
     }
     static __device__ __forceinline__ void add(acc& P, const acc& Q) { ed::add(P, Q); }
     static __device__ __forceinline__ void add4_mem(acc& P, const uint4* q, fe* sh, int l) {
@@ -1477,19 +1480,19 @@ __global__ void __launch_bounds__(128, M::kAccBlocks) k_accumulate_batched(const
     }
 }
 
-// The block's sum of m points at `in`, four lanes per addition: group g of the block's
-// 32 groups sums in[g], in[g + 32], ... in sequence, then a tree over the groups in
-// shared memory (depth ceil(m / 32) - 1 + 5 four-lane additions). Every group of a warp
-// runs the same additions (a missing operand is the identity; idle groups of warp 0 add
-// and discard), so each __syncwarp inside them is warp-wide; a warp with no active
-// group skips a level as a whole. Thread 0 stores the sum.
+// The block's sum of m points. More than 128 are first summed to 128, one thread each;
+// then the block's 32 groups of four lanes sum points g, g + 32, ... in sequence, four
+// lanes per addition, and a tree over the groups in shared memory ends it (5 levels).
+// Every group of a warp runs the same additions (a missing operand is the identity; idle
+// groups of warp 0 add and discard), so each __syncwarp inside them is warp-wide; a warp
+// with no active group skips a level as a whole. Thread 0 stores the sum.
 constexpr int kTreeThreads = 128;
 constexpr int kTreeGroups = kTreeThreads / 4;
 constexpr size_t kTreeWave = 152 * 3;  // blocks resident at once (3 per SM)
 
 template <class M>
 struct TreeShared {
-    uint4 pub[kTreeGroups * kXyzzVec];
+    uint4 pub[kTreeThreads * kXyzzVec];
     uint4 idn[kXyzzVec];
     fe sh[kTreeGroups][4];
 };
@@ -1504,17 +1507,27 @@ __device__ __forceinline__ void tree_init(TreeShared<M>& s) {
     __syncthreads();
 }
 
-template <class M>
-__device__ __forceinline__ void block_sum(TreeShared<M>& s, const uint4* __restrict__ in, uint32_t m, uint4* __restrict__ out) {
+// src(i): the address of point i, or of the identity s.idn.
+template <class M, class Src>
+__device__ __forceinline__ void block_sum_of(TreeShared<M>& s, const Src& src, uint32_t m, uint4* __restrict__ out) {
     const int t = threadIdx.x, g = t >> 2, l = t & 3, warp = t >> 5;
     typename M::acc acc;
-    if ((uint32_t)g < m)
-        M::load(acc, in + (size_t)g * kXyzzVec);
-    else
-        M::set_inf(acc);
-    for (uint32_t i0 = kTreeGroups; i0 < m; i0 += kTreeGroups) {
-        const uint32_t i = i0 + g;
-        M::add4_mem(acc, i < m ? in + (size_t)i * kXyzzVec : s.idn, s.sh[g], l);
+    if (m > kTreeThreads) {   // first by threads, a point of every 128 each
+        M::load(acc, src(t));
+        for (uint32_t i = t + kTreeThreads; i < m; i += kTreeThreads) M::add_mem(acc, src(i));
+        M::store(s.pub + t * kXyzzVec, acc);
+        __syncthreads();
+        m = kTreeThreads;
+        M::load(acc, s.pub + g * kXyzzVec);
+        for (uint32_t i = kTreeGroups + g; i < kTreeThreads; i += kTreeGroups)
+            M::add4_mem(acc, s.pub + i * kXyzzVec, s.sh[g], l);
+        __syncthreads();      // the points are read before the levels below publish over them
+    } else {
+        M::load(acc, (uint32_t)g < m ? src(g) : s.idn);
+        for (uint32_t i0 = kTreeGroups; i0 < m; i0 += kTreeGroups) {
+            const uint32_t i = i0 + g;
+            M::add4_mem(acc, i < m ? src(i) : s.idn, s.sh[g], l);
+        }
     }
     // level h: groups [h, 2h) publish, groups [0, h) add them. The slots read at
     // level h, [h, 2h), are never written at a later level (those write [h', 2h')
@@ -1530,6 +1543,11 @@ __device__ __forceinline__ void block_sum(TreeShared<M>& s, const uint4* __restr
         }
     }
     if (t == 0) M::store(out, acc);
+}
+
+template <class M>
+__device__ __forceinline__ void block_sum(TreeShared<M>& s, const uint4* __restrict__ in, uint32_t m, uint4* __restrict__ out) {
+    block_sum_of(s, [&](uint32_t i) { return in + (size_t)i * kXyzzVec; }, m, out);
 }
 
 __device__ __forceinline__ uint4* merge_dest(uint4* parts, uint4* buckets, uint32_t d) {
@@ -1568,7 +1586,8 @@ __global__ void __launch_bounds__(kTreeThreads) k_merge_parts(uint4* parts, uint
 
 // ---------------------------------------------------------------- stage 6
 
-// Thread (wi, g): Y = sum_{i=1..L} B[gL+i], V = sum_{i=1..L} i * B[gL+i] (bucket b at index b-1).
+// Thread (wi, g): Y = sum_{i=1..L} B[gL+i], V = sum_{i=1..L} i * B[gL+i] (bucket b at
+// index b-1): 2 (L - 1) additions.
 template <class M>
 __global__ void __launch_bounds__(128) k_reduce_segments(const uint4* __restrict__ buckets, uint32_t Bp, uint32_t L, int w0, int nwin,
                                   uint32_t G, uint4* __restrict__ Y, uint4* __restrict__ V) {
@@ -1577,9 +1596,13 @@ __global__ void __launch_bounds__(128) k_reduce_segments(const uint4* __restrict
     const size_t wi = id / G, g = id % G;
     const uint4* seg = buckets + ((size_t)(w0 + wi) * Bp + g * L) * kXyzzVec;
     typename M::acc T, S;
-    M::set_inf(T);
-    M::set_inf(S);
-    for (int i = (int)L; i >= 1; --i) {
+    const uint4* last = seg + (size_t)(L - 1) * kXyzzVec;
+    if (M::empty(last))
+        M::set_inf(T);
+    else
+        M::load(T, last);
+    S = T;
+    for (int i = (int)L - 1; i >= 1; --i) {
         M::add_mem(T, seg + (size_t)(i - 1) * kXyzzVec);   // T += B
         M::add(S, T);                                       // S += T
     }
@@ -1587,50 +1610,48 @@ __global__ void __launch_bounds__(128) k_reduce_segments(const uint4* __restrict
     M::store(V + id * kXyzzVec, S);
 }
 
-// Thread (wi, k, q): partial of Z_k = sum_{g: bit k of g set} Y_g over the q-th of Q
-// equal slices of those G/2 indices, or for k == logG the partial of sum_g V_g over
-// the q-th slice of all G indices. The j-th index with bit k set is j with a one
-// inserted at bit k, so the threads of a warp (same k) run the same additions.
-template <class M>
-__global__ void k_bitsums(const uint4* __restrict__ Y, const uint4* __restrict__ V, int nwin, uint32_t G,
-                          int logG, uint32_t Q, uint4* __restrict__ P) {
-    const size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    const size_t per_w = (size_t)(logG + 1) * Q;
-    if (id >= (size_t)nwin * per_w) return;
-    const size_t wi = id / per_w;
-    const int kk = (int)((id % per_w) / Q);
-    const int k = kk == 0 ? logG : kk - 1;  // the V slices (twice as long) are scheduled first
-    const uint32_t q = (uint32_t)(id % Q);
-    typename M::acc acc;
-    M::set_inf(acc);
-    if (k == logG) {
-        const uint32_t span = G / Q, g0 = q * span;
-        for (uint32_t g = g0; g < g0 + span; ++g) M::add_mem(acc, V + (wi * G + g) * kXyzzVec);
+// Sums of the segments' points by the bits of their index, four lanes per addition.
+// Per window there are (logG + 2) nb blocks: block (k, q), k < logG, sums the q-th of nb
+// equal slices of the G/2 points Y_g with bit k of g set (the j-th such index is j with
+// a one inserted at bit k); the last 2 nb blocks sum slices of all V_g. Every block
+// sums (G/2) / nb points (block_sum_of). What bounds it is the latency of its additions:
+// 5.7 (Edwards) or 11 us (XYZZ) each on four lanes while the blocks fit two per SM, about
+// twice that on one thread. One thread per slice of eight points and a launch of block
+// trees over the slices took 87 + 29 us where this takes 51 + 8 (Edwards, 13 windows of 512
+// buckets) and 145 + 68 us where this takes 78 (XYZZ, 32 windows of 256). kRaw:
+// Y = V are the buckets themselves (L = 1), which may be empty.
+template <class M, bool kRaw>
+__global__ void __launch_bounds__(kTreeThreads) k_bit_sums(const uint4* __restrict__ Y, const uint4* __restrict__ V, int nwin,
+                                                          uint32_t G, int logG, uint32_t nb, uint4* __restrict__ P) {
+    __shared__ TreeShared<M> s;
+    const uint32_t per_w = (uint32_t)(logG + 2) * nb;
+    const uint32_t wi = blockIdx.x / per_w, r = blockIdx.x % per_w;
+    if (wi >= (uint32_t)nwin) return;  // whole block
+    tree_init(s);
+    const uint32_t k = r / nb;
+    auto at_point = [&](const uint4* q) { return kRaw && M::empty(q) ? (const uint4*)s.idn : q; };
+    if (k < (uint32_t)logG) {
+        const uint32_t span = (G / 2) / nb, j0 = (r % nb) * span, low = (1u << k) - 1u;
+        const uint4* y = Y + (size_t)wi * G * kXyzzVec;
+        block_sum_of(s, [&](uint32_t i) {
+            const uint32_t j = j0 + i, g = ((j & ~low) << 1) | (1u << k) | (j & low);
+            return at_point(y + (size_t)g * kXyzzVec);
+        }, span, P + (size_t)blockIdx.x * kXyzzVec);
     } else {
-        const uint32_t span = (G / 2) / Q, j0 = q * span, low = (1u << k) - 1u;
-        for (uint32_t j = j0; j < j0 + span; ++j) {
-            const uint32_t g = ((j & ~low) << 1) | (1u << k) | (j & low);
-            M::add_mem(acc, Y + (wi * G + g) * kXyzzVec);
-        }
+        const uint32_t v = r - (uint32_t)logG * nb;                     // slice of 2 nb
+        const uint32_t g0 = (uint32_t)((uint64_t)v * G / (2 * nb)), g1 = (uint32_t)((uint64_t)(v + 1) * G / (2 * nb));
+        const uint4* x = V + ((size_t)wi * G + g0) * kXyzzVec;
+        block_sum_of(s, [&](uint32_t i) { return at_point(x + (size_t)i * kXyzzVec); }, g1 - g0,
+                     P + (size_t)blockIdx.x * kXyzzVec);
     }
-    M::store(P + (wi * per_w + (size_t)k * Q + q) * kXyzzVec, acc);
 }
 
-// Block (s, b) sums in[s][F 32 b .. F 32 (b + 1) - 1] (within the segment's m points)
-// into out[s][b]; a segment of m points needs log_(32 F) m launches. F is chosen so that
-// a launch fills about one wave of blocks.
+// Block seg: out[seg] = the sum of in[seg][0 .. m - 1].
 template <class M>
-__global__ void __launch_bounds__(kTreeThreads) k_sum_tree(const uint4* __restrict__ in, size_t nseg, uint32_t m,
-                                                          uint32_t F, uint4* __restrict__ out) {
+__global__ void __launch_bounds__(kTreeThreads) k_sum_rows(const uint4* __restrict__ in, uint32_t m, uint4* __restrict__ out) {
     __shared__ TreeShared<M> s;
-    const uint32_t per = kTreeGroups * F;
-    const uint32_t nb = (m + per - 1) / per;
-    const size_t seg = blockIdx.x / nb;
-    const uint32_t b = blockIdx.x % nb;
-    if (seg >= nseg) return;  // whole block
     tree_init(s);
-    const uint32_t left = m - b * per;
-    block_sum(s, in + (seg * m + (size_t)b * per) * kXyzzVec, left < per ? left : per, out + (seg * nb + b) * kXyzzVec);
+    block_sum(s, in + (size_t)blockIdx.x * m * kXyzzVec, m, out + (size_t)blockIdx.x * kXyzzVec);
 }
 
 // ---------------------------------------------------------------- stage 7
@@ -1640,8 +1661,8 @@ __global__ void __launch_bounds__(kTreeThreads) k_sum_tree(const uint4* __restri
 // level) and each product over the lanes of its warp (wred.cuh). The next operand's
 // loads are issued before the current operation, so they overlap it.
 
-// Block w: S_w = L sum_{k < logG} 2^k Z_k + Z_logG for window w, by Horner from the
-// top term; S_w is left in the chain's operand form (limbs).
+// Block w: S_w = L sum_{k < logG} 2^k Z_k + Z_logG + Z_(logG + 1) for window w (the last
+// two: the halves of sum_g V_g), by Horner from the top term; S_w is left in the chain's operand form (limbs).
 template <class M>
 __global__ void __launch_bounds__(128, 1) k_window_horner_w(const uint4* __restrict__ Z, int nwin, int logG, int log2L,
                                                          int* __restrict__ S) {
@@ -1652,7 +1673,7 @@ __global__ void __launch_bounds__(128, 1) k_window_horner_w(const uint4* __restr
     wred::Group g;
     wred::init(g, mem);
     C::load_const(g);
-    const uint32_t* z = reinterpret_cast<const uint32_t*>(Z + (size_t)w * (logG + 1) * kXyzzVec);
+    const uint32_t* z = reinterpret_cast<const uint32_t*>(Z + (size_t)w * (logG + 2) * kXyzzVec);
     constexpr size_t kWords = 4 * kXyzzVec;
     C::set_inf(g);
     wred::Packed next = wred::load_packed(g, z + (size_t)(logG > 0 ? logG - 1 : logG) * kWords);
@@ -1664,8 +1685,12 @@ __global__ void __launch_bounds__(128, 1) k_window_horner_w(const uint4* __restr
         C::add(g);
     }
     for (int t = 0; t < log2L; ++t) C::dbl(g, t == log2L - 1);
-    C::set_operand(g, next.limb, wred::zero_z(g, next));   // Z_logG
-    C::add(g);
+    for (int h = 0; h < 2; ++h) {
+        const wred::Packed q = next;   // Z_(logG + h)
+        if (h == 0) next = wred::load_packed(g, z + (size_t)(logG + 1) * kWords);
+        C::set_operand(g, q.limb, wred::zero_z(g, q));
+        C::add(g);
+    }
     const int v = C::as_operand(g);
     if (g.lane < 16) S[(size_t)w * wred::kLimbPointWords + 16 * g.w + g.lane] = v;
 }
@@ -1712,7 +1737,8 @@ struct Plan {
     size_t max_pieces, max_parts, max_small, max_tree[3];   // per group: bounds over any digits
     int gw;         // windows per group
     int ngroups;
-    uint32_t L, G, Q;
+    uint32_t L, G;
+    uint32_t nb;     // blocks per bit of the segment sums
     int logG, log2L;
     size_t off_status, off_ctrl, ctrl_bytes;   // status words, then the groups' counters: cleared together
     size_t off_points, off_keys0, off_vals0, off_keys1, off_vals1, off_rank, off_hist, off_dtot;
@@ -1725,7 +1751,6 @@ struct Plan {
     size_t off_S, total;
 };
 
-constexpr uint64_t kReduceThreads = 32768;
 
 int ilog2(uint64_t v) {
     int r = 0;
@@ -1875,19 +1900,47 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool allow_groups = true) {
         p->max_tree[1] = p->max_tree[2] = multi / kTreeParts + 1;
         if (p->max_parts >= kPart || p->max_pieces >= (1ull << 32)) return false;
     }
-    // bucket reduction geometry: segments of L buckets, the longest L that still
-    // leaves kReduceThreads level-1 threads over all windows (longer segments mean
-    // fewer segment sums for the bit-sum stage, but fewer threads for the running sums)
-    uint64_t group_buckets = (uint64_t)p->W * p->Bp;
-    uint32_t L = 2;
-    const uint64_t reduce_threads = tr > 0 ? (1ull << tr) : kReduceThreads;
-    while (L < p->Bp && group_buckets / (2 * L) >= reduce_threads) L <<= 1;
-    if (L > p->Bp) L = p->Bp;
-    p->L = L;
-    p->G = p->Bp / L;
+    // Bucket reduction: segments of L buckets summed by a thread each (2 (L - 1)
+    // additions in sequence), then blocks of four-lane additions over the W G segment
+    // sums (k_bit_sums). L is the power of two with the least estimated time, from the
+    // measured time of one addition alone and of one per resident thread with the GPU
+    // full: 10.5 and 25 us on one thread (Edwards; XYZZ 18 and 29 us), 5.7 and 7.5 us (11 and
+    // 24 us) on four lanes with three blocks per SM. Small calls take L = 1 or 2, 2^19 buckets L = 16.
+    {
+        const double t1 = p->edw ? 10.5 : 18.0, t1_full = p->edw ? 25.0 : 29.0;
+        const double t4 = p->edw ? 5.7 : 11.0, t4_full = p->edw ? 7.5 : 24.0;
+        double best = 0;
+        p->L = 0;
+        for (uint32_t L = 1; L <= p->Bp; L <<= 1) {
+            const uint32_t G = p->Bp / L;
+            const int lg = ilog2(G);
+            const size_t per_nb = (size_t)p->gw * (lg + 2);
+            const double threads = (double)p->gw * G / (double)kWave;
+            const double add1 = t1 > t1_full * threads ? t1 : t1_full * threads;
+            // a tuned number of segments: the longest L that leaves as many
+            const bool forced = tr > 0;
+            if (forced && L > 1 && (uint64_t)p->W * G < (1ull << tr)) break;
+            if (forced) p->L = 0;
+            for (uint32_t nb = 1; nb == 1 || (per_nb * nb <= kTreeWave && G / 2 / nb >= (uint32_t)kTreeGroups); nb <<= 1) {
+                const double blocks = (double)(per_nb * nb) / (double)kTreeWave;
+                const double in_blocks = blocks * kTreeWave * kTreeThreads / (double)kWave;
+                const uint32_t span = G / 2 / nb, by_thread = span > kTreeThreads ? span / kTreeThreads - 1 : 0;
+                const double steps = (double)((span < kTreeThreads ? span : kTreeThreads) + kTreeGroups - 1) / kTreeGroups + 4;
+                const double t = 2.0 * (L - 1) * add1 + (L > 1 ? 3.0 : 0.0) +
+                                 by_thread * (t1 > t1_full * in_blocks ? t1 : t1_full * in_blocks) +
+                                 steps * (t4 > t4_full * blocks ? t4 : t4_full * blocks) +
+                                 (nb > 1 ? 3.0 + t4 * ilog2(nb) : 0.0);
+                if (p->L == 0 || t < best) {
+                    best = t;
+                    p->L = L;
+                    p->nb = nb;
+                }
+            }
+        }
+    }
+    p->G = p->Bp / p->L;
     p->logG = ilog2(p->G);
-    p->log2L = ilog2(L);
-    p->Q = p->G >= 8 ? p->G / 8 : 1;
+    p->log2L = ilog2(p->L);
     // workspace layout, 256-byte aligned pieces
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -1918,11 +1971,12 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool allow_groups = true) {
     p->off_pieces = take(p->ngroups * p->max_pieces * 16);
     p->off_small = take(p->ngroups * p->max_small * 16);
     for (int k = 0; k < 3; ++k) p->off_tree[k] = take(p->ngroups * p->max_tree[k] * 16);
-    p->off_Y = take((size_t)p->ngroups * p->gw * p->G * XY);    // per group
-    p->off_V = take((size_t)p->ngroups * p->gw * p->G * XY);
-    const size_t zs = (size_t)p->gw * (p->logG + 1) * p->Q;
-    p->off_P0 = take((size_t)p->ngroups * zs * XY);
-    p->off_P1 = take((size_t)p->ngroups * zs * XY);
+    const size_t segs = p->L > 1 ? (size_t)p->ngroups * p->gw * p->G : 0;   // per group
+    p->off_Y = take(segs * XY);
+    p->off_V = take(segs * XY);
+    const size_t zs = (size_t)p->ngroups * p->gw * (p->logG + 2);
+    p->off_P0 = take(zs * p->nb * XY);
+    p->off_P1 = take(p->nb > 1 ? zs * XY : 0);
     p->off_S = take((size_t)p->W * wred::kLimbPointWords * sizeof(int));
     p->total = off;
     return true;
@@ -2222,12 +2276,6 @@ int enqueue_head(const Plan& p, const uint32_t* points, const uint32_t* scalars,
 // partial merges, bucket reduction, and S_w for each window, in the group's buffers.
 template <class M>
 int enqueue_group_tail_m(const Plan& p, const AccArgs& acc, int g, void* workspace, cudaStream_t s) {
-    const size_t yv = (size_t)p.gw * p.G * kXyzzVec;
-    const size_t zs = (size_t)p.gw * (p.logG + 1) * p.Q * kXyzzVec;
-    uint4* Y = at<uint4>(workspace, p.off_Y) + (size_t)g * yv;
-    uint4* V = at<uint4>(workspace, p.off_V) + (size_t)g * yv;
-    uint4* P0 = at<uint4>(workspace, p.off_P0) + (size_t)g * zs;
-    uint4* P1 = at<uint4>(workspace, p.off_P1) + (size_t)g * zs;
     int* S = at<int>(workspace, p.off_S);
     const PieceArgs a = piece_args(p, workspace, g);
     // 5. the parts of buckets cut into pieces, as many tree levels as a bucket can need
@@ -2241,27 +2289,29 @@ int enqueue_group_tail_m(const Plan& p, const AccArgs& acc, int g, void* workspa
         note_launches(1);
     }
     // 6. bucket reduction of the group's windows
-    const size_t WG = (size_t)a.nwin * p.G;
-    k_reduce_segments<M><<<grid_for(WG, 128), 128, 0, s>>>(a.buckets, p.Bp, p.L, a.w0, a.nwin, p.G, Y, V);
-    const size_t nseg = (size_t)a.nwin * (p.logG + 1);
-    k_bitsums<M><<<grid_for(nseg * p.Q, 128), 128, 0, s>>>(Y, V, a.nwin, p.G, p.logG, p.Q, P0);
-    note_launches(2);
-    uint32_t m = p.Q;
-    uint4* zin = P0;
-    uint4* zout = P1;
-    while (m > 1) {
-        uint32_t F = 2;  // per-group fan-in: about one wave of blocks, at most 8 sequential additions
-        while (F < 8 && nseg * ((m + kTreeGroups * F - 1) / (kTreeGroups * F)) > kTreeWave) F <<= 1;
-        const uint32_t nb = (m + kTreeGroups * F - 1) / (kTreeGroups * F);
-        k_sum_tree<M><<<(unsigned)(nseg * nb), kTreeThreads, 0, s>>>(zin, nseg, m, F, zout);
+    const size_t nseg = (size_t)a.nwin * (p.logG + 2);
+    uint4* P0 = at<uint4>(workspace, p.off_P0) + (size_t)g * p.gw * (p.logG + 2) * p.nb * kXyzzVec;
+    uint4* Z = P0;
+    if (p.L > 1) {
+        const size_t yv = (size_t)p.gw * p.G * kXyzzVec;
+        uint4* Y = at<uint4>(workspace, p.off_Y) + (size_t)g * yv;
+        uint4* V = at<uint4>(workspace, p.off_V) + (size_t)g * yv;
+        k_reduce_segments<M><<<grid_for((size_t)a.nwin * p.G, 128), 128, 0, s>>>(a.buckets, p.Bp, p.L, a.w0, a.nwin, p.G,
+                                                                                Y, V);
+        k_bit_sums<M, false><<<(unsigned)(nseg * p.nb), kTreeThreads, 0, s>>>(Y, V, a.nwin, p.G, p.logG, p.nb, P0);
+        note_launches(2);
+    } else {
+        const uint4* B = a.buckets + (size_t)a.w0 * p.Bp * kXyzzVec;
+        k_bit_sums<M, true><<<(unsigned)(nseg * p.nb), kTreeThreads, 0, s>>>(B, B, a.nwin, p.G, p.logG, p.nb, P0);
         note_launches(1);
-        m = nb;
-        uint4* tmp = zin;
-        zin = zout;
-        zout = tmp;
+    }
+    if (p.nb > 1) {
+        Z = at<uint4>(workspace, p.off_P1) + (size_t)g * p.gw * (p.logG + 2) * kXyzzVec;
+        k_sum_rows<M><<<(unsigned)nseg, kTreeThreads, 0, s>>>(P0, p.nb, Z);
+        note_launches(1);
     }
     // 7a. the per-window sums S_w
-    k_window_horner_w<M><<<(unsigned)a.nwin, 128, 0, s>>>(zin, a.nwin, p.logG, p.log2L, S + (size_t)a.w0 * wred::kLimbPointWords);
+    k_window_horner_w<M><<<(unsigned)a.nwin, 128, 0, s>>>(Z, a.nwin, p.logG, p.log2L, S + (size_t)a.w0 * wred::kLimbPointWords);
     note_launches(1);
     return check_launch("msm tail");
 }

@@ -50,3 +50,20 @@ def test_longest_pieces(edwards):
         assert g1.from_limbs(pkg.to_host(out)) == closed_form_limbs(s, a)
     finally:
         pkg.msm_g1_set_schedule(k, edwards=edwards)
+
+
+@pytest.mark.parametrize("edwards", [False, True])
+@pytest.mark.parametrize("c,reduce_log2", [(2, 8), (5, 8), (8, 8), (8, 13), (11, 8), (11, 12), (11, 20), (14, 10), (14, 17)])
+def test_bucket_reduction_geometries(edwards, c, reduce_log2):
+    """Segments of one to hundreds of buckets, most of them empty, in every split over blocks."""
+    n = 300
+    a, s, pts = msm_inputs(8400, tag=71)
+    a, s, pts = a[:n], s[:n], pts[:n]
+    k = n.bit_length() - 1
+    pkg.msm_g1_set_schedule(k, 0, 0, 0, reduce_log2, 0, edwards=edwards)
+    try:
+        out = pkg.msm_g1(pkg.to_device(pts), pkg.to_device(a), c=c, scalar_bits=253, edwards=edwards)
+        torch.cuda.synchronize()
+        assert g1.from_limbs(pkg.to_host(out)) == closed_form_limbs(s, a)
+    finally:
+        pkg.msm_g1_set_schedule(k, edwards=edwards)
