@@ -1772,12 +1772,31 @@ int table_mode(uint32_t flags) {
            ((flags & MSM377_PRECOMPUTED) ? 4 : 0);
 }
 
-int default_c(size_t n, int sgn, uint32_t flags) {
+// Window width by floor(log2 n) for signed digits, per mode (bit 0 Edwards, bit 1 GLV):
+// the fastest of the widths 4..17 measured on GB300 at 1.05 and 1.55 times each power of
+// two (the better of the two on average). A wider window means fewer windows but more
+// buckets; which widths pay also depends on the top window, which is short (and its
+// few buckets heavy) when c just fails to divide the scalar's bits: with GLV's 127-bit
+// halves 11 and 16 divide well, so n = 2^16 .. 2^22 takes 16 (n = 2.7 * 10^5, Edwards + GLV:
+// c = 14 1949, 15 1742, 16 1616, 17 1858 us) and 2^12 .. 2^14 takes 11.
+constexpr int kDefaultLogs = 23;
+constexpr int8_t kDefaultC[4][kDefaultLogs] = {
+    {4, 4, 4, 4, 4, 4, 6, 6, 7, 7, 8, 11, 8, 11, 11, 13, 13, 15, 15, 16, 16, 17, 17},   // XYZZ
+    {4, 4, 4, 4, 4, 4, 5, 5, 6, 7, 8, 8, 11, 11, 11, 11, 14, 15, 15, 16, 16, 17, 17},   // Edwards
+    {4, 4, 4, 4, 4, 4, 4, 4, 4, 4, 9, 10, 11, 11, 11, 14, 15, 16, 16, 16, 17, 17, 17},  // XYZZ + GLV
+    {4, 4, 4, 4, 4, 4, 4, 4, 5, 5, 5, 8, 11, 11, 11, 12, 15, 16, 16, 16, 16, 16, 16}};  // Edwards + GLV
+
+// single: one call on its own, whose latency counts. The jobs of a batch overlap, so their
+// total work counts, and there the rule by size below is the better one (24 jobs of 2^10
+// to 2^18 points: 7.25 ms, 7.33 with the table).
+int default_c(size_t n, int sgn, uint32_t flags, bool single = true) {
     int lg = n > 1 ? ilog2(n) : 0;
     if (sgn && lg < 32) {
         const int t = g_ctable[table_mode(flags)][lg].load(std::memory_order_relaxed);
         if (t > 0) return t;
     }
+    if (single && sgn && !(flags & MSM377_PRECOMPUTED))
+        return kDefaultC[table_mode(flags) & 3][lg < kDefaultLogs ? lg : kDefaultLogs - 1];
     if (flags & MSM377_GLV) ++lg;  // 2n points per window
     if (flags & MSM377_PRECOMPUTED) lg += 2;  // one bucket set for all windows: wider windows pay
     int c = lg - 4;
@@ -1789,8 +1808,8 @@ int default_c(size_t n, int sgn, uint32_t flags) {
 
 constexpr int kMaxGroups = 8;
 
-// allow_groups = false: one window group (batched calls overlap whole jobs instead).
-bool make_plan(size_t n, const msm_opts* o, Plan* p, bool allow_groups = true) {
+// single = false (batched calls): one window group; whole jobs overlap instead.
+bool make_plan(size_t n, const msm_opts* o, Plan* p, bool single = true) {
     if (!o) return false;
     p->n = n;
     p->edw = (o->flags & MSM377_EDWARDS) ? 1 : 0;
@@ -1803,7 +1822,7 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool allow_groups = true) {
     p->user_bits = o->scalar_bits ? o->scalar_bits : 256;
     if (p->user_bits < 1 || p->user_bits > 256) return false;
     p->bits = p->glv ? 127 : p->user_bits;  // GLV halves are below 2^127
-    p->c = o->c ? o->c : default_c(n, p->sgn, o->flags);
+    p->c = o->c ? o->c : default_c(n, p->sgn, o->flags, single);
     if (p->c < 2 || p->c > 20) return false;
     if (n >= (1ull << 30)) return false;
     const size_t np = p->glv ? 2 * n : n;
@@ -1859,7 +1878,7 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool allow_groups = true) {
     // 2^22 20.7 / 22.0 / 22.6 ms -- the overlapped tails slow the accumulation more
     // than they save, so the autotuner keeps one group at every size measured.
     int groups = 1;
-    if (allow_groups && !p->pre) {
+    if (single && !p->pre) {
         groups = tg > 0 ? tg : 1;
         if (groups > p->W) groups = p->W;
         if (groups > kMaxGroups) groups = kMaxGroups;
