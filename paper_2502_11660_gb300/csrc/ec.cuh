@@ -108,26 +108,23 @@ __device__ __forceinline__ void dbl(xyzz& P) {
 // U2 = x2 ZZ1, S2 = y2 ZZZ1, Pd = U2 - X1, R = S2 - Y1, PP = Pd^2, PPP = Pd PP,
 // Q1 = X1 PP, X3 = R^2 - PPP - 2 Q1, Y3 = R (Q1 - X3) - Y1 PPP,
 // ZZ3 = ZZ1 PP, ZZZ3 = ZZZ1 PPP.
-__device__ __forceinline__ void madd(xyzz& P, bool& p_inf, const affine& Q) {
-    if (is_inf(Q)) return;
+// madd_but_double leaves P = Q undone and returns true: the caller doubles Q.
+__device__ __forceinline__ bool madd_but_double(xyzz& P, bool& p_inf, const affine& Q) {
+    if (is_inf(Q)) return false;
     if (p_inf) {
         from_affine(P, Q);
         p_inf = false;
-        return;
+        return false;
     }
     fe U2, S2, Pd, R;
     fq::mul2(U2, Q.x, P.ZZ, S2, Q.y, P.ZZZ);
     fq::sub(Pd, U2, P.X);
     fq::sub(R, S2, P.Y);
     if (fq::is_zero(Pd)) {
-        if (fq::is_zero(R)) {
-            mdbl(P, Q);
-            p_inf = is_inf(P);
-        } else {
-            set_inf(P);
-            p_inf = true;
-        }
-        return;
+        if (fq::is_zero(R)) return true;
+        set_inf(P);
+        p_inf = true;
+        return false;
     }
     fe PP, PPP, Q1, t;
     fq::mul2(PP, Pd, Pd, t, R, R);              // PP, R^2
@@ -139,6 +136,14 @@ __device__ __forceinline__ void madd(xyzz& P, bool& p_inf, const affine& Q) {
     fq::sub(t, Q1, P.X);
     fq::mul2(PPP, P.Y, PPP, t, R, t);           // Y1 PPP, R (Q1 - X3)
     fq::sub(P.Y, t, PPP);
+    return false;
+}
+
+__device__ __forceinline__ void madd(xyzz& P, bool& p_inf, const affine& Q) {
+    if (madd_but_double(P, p_inf, Q)) {
+        mdbl(P, Q);
+        p_inf = is_inf(P);
+    }
 }
 
 __device__ __forceinline__ void madd(xyzz& P, const affine& Q) {
