@@ -99,8 +99,7 @@ int fq_to_montgomery(const uint32_t *in, uint32_t *out, size_t n, void *stream);
  *   MSM377_FQMUL_WARP      a b 2^-384 mod p with one warp per product: lane j holds
  *                          limb j, three column products (a b, the Montgomery
  *                          quotient, its multiple of p) with warp-wide carry
- *                          resolution; the low-latency form the MSM's window chains
- *                          use. Operands may be any values below 8p here.
+ *                          resolution. Operands may be any values below 8p here.
  *   MSM377_FQMUL_PAPER     the paper's own format and reduction (Sec. III-B .. III-E)
  *                          on standard-form operands below 6p (the unreduced operands
  *                          of its final multiplications): 16 elements of 25 bits,

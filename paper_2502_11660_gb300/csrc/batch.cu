@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kPaddBlock, kPaddPerSm) k_padd(const uint32_t*
                 fq::to_mont(P.ZZZ, P.ZZZ);
             }
             bool inf = ec::is_inf(P);
-            dbl = ec::madd_but_double(P, inf, Q);
+            dbl = ec::madd_but_double<false>(P, inf, Q);
             if (!dbl) store_padd(out, i, n, P, form);
         }
         const uint32_t m = __ballot_sync(0xffffffffu, dbl);

@@ -238,79 +238,47 @@ struct MontAccD {
     uint32_t e[14], o[14];
 };
 
-__device__ __forceinline__ void mont_dstep(MontAccD& t, uint32_t x0, uint32_t x1, const uint32_t* b, uint32_t neg1) {
+// a[0..11] += x (b_0 + 2^64 b_1 + ... ), six products whose low and high halves sit in
+// adjacent words; kTail: the carry goes on into a[12], a[13], else none leaves a[11].
+template <bool kTail>
+__device__ __forceinline__ void mad_chain(uint32_t* a, uint32_t x, const uint32_t (&b)[6]) {
+    if constexpr (kTail) {
+    asm("mad.lo.cc.u32 %0, %14, %15, %0;\n\tmadc.hi.cc.u32 %1, %14, %15, %1;\n\t"
+        "madc.lo.cc.u32 %2, %14, %16, %2;\n\tmadc.hi.cc.u32 %3, %14, %16, %3;\n\t"
+        "madc.lo.cc.u32 %4, %14, %17, %4;\n\tmadc.hi.cc.u32 %5, %14, %17, %5;\n\t"
+        "madc.lo.cc.u32 %6, %14, %18, %6;\n\tmadc.hi.cc.u32 %7, %14, %18, %7;\n\t"
+        "madc.lo.cc.u32 %8, %14, %19, %8;\n\tmadc.hi.cc.u32 %9, %14, %19, %9;\n\t"
+        "madc.lo.cc.u32 %10, %14, %20, %10;\n\tmadc.hi.cc.u32 %11, %14, %20, %11;\n\t"
+        "addc.cc.u32 %12, %12, 0;\n\taddc.u32 %13, %13, 0;"
+        : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
+          "+r"(a[8]), "+r"(a[9]), "+r"(a[10]), "+r"(a[11]), "+r"(a[12]), "+r"(a[13])
+        : "r"(x), "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3]), "r"(b[4]), "r"(b[5]));
+    } else {
+    asm("mad.lo.cc.u32 %0, %12, %13, %0;\n\tmadc.hi.cc.u32 %1, %12, %13, %1;\n\t"
+        "madc.lo.cc.u32 %2, %12, %14, %2;\n\tmadc.hi.cc.u32 %3, %12, %14, %3;\n\t"
+        "madc.lo.cc.u32 %4, %12, %15, %4;\n\tmadc.hi.cc.u32 %5, %12, %15, %5;\n\t"
+        "madc.lo.cc.u32 %6, %12, %16, %6;\n\tmadc.hi.cc.u32 %7, %12, %16, %7;\n\t"
+        "madc.lo.cc.u32 %8, %12, %17, %8;\n\tmadc.hi.cc.u32 %9, %12, %17, %9;\n\t"
+        "madc.lo.cc.u32 %10, %12, %18, %10;\n\tmadc.hi.u32 %11, %12, %18, %11;"
+        : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
+          "+r"(a[8]), "+r"(a[9]), "+r"(a[10]), "+r"(a[11])
+        : "r"(x), "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3]), "r"(b[4]), "r"(b[5]));
+    }
+}
+
+// The rows x0 b and x1 b of a step.
+__device__ __forceinline__ void mont_rows(MontAccD& t, uint32_t x0, uint32_t x1, const uint32_t* b) {
+    const uint32_t even[6] = {b[0], b[2], b[4], b[6], b[8], b[10]}, odd[6] = {b[1], b[3], b[5], b[7], b[9], b[11]};
+    mad_chain<true>(t.e, x0, even);
+    mad_chain<true>(t.o, x0, odd);
+    mad_chain<true>(t.o, x1, even);
+    mad_chain<false>(t.e + 2, x1, odd);   // no carry leaves E[13]
+}
+
+// The two quotient digits of a step, their rows, and the shift by two limbs.
+__device__ __forceinline__ void mont_digits(MontAccD& t, uint32_t neg1) {
     uint32_t* E = t.e;
     uint32_t* O = t.o;
-    // E[0..11] += x0 b_even, carry into E[12..13]
-    asm("mad.lo.cc.u32 %0, %14, %15, %0;\n\t"
-        "madc.hi.cc.u32 %1, %14, %15, %1;\n\t"
-        "madc.lo.cc.u32 %2, %14, %16, %2;\n\t"
-        "madc.hi.cc.u32 %3, %14, %16, %3;\n\t"
-        "madc.lo.cc.u32 %4, %14, %17, %4;\n\t"
-        "madc.hi.cc.u32 %5, %14, %17, %5;\n\t"
-        "madc.lo.cc.u32 %6, %14, %18, %6;\n\t"
-        "madc.hi.cc.u32 %7, %14, %18, %7;\n\t"
-        "madc.lo.cc.u32 %8, %14, %19, %8;\n\t"
-        "madc.hi.cc.u32 %9, %14, %19, %9;\n\t"
-        "madc.lo.cc.u32 %10, %14, %20, %10;\n\t"
-        "madc.hi.cc.u32 %11, %14, %20, %11;\n\t"
-        "addc.cc.u32 %12, %12, 0;\n\t"
-        "addc.u32 %13, %13, 0;"
-        : "+r"(E[0]), "+r"(E[1]), "+r"(E[2]), "+r"(E[3]), "+r"(E[4]), "+r"(E[5]), "+r"(E[6]), "+r"(E[7]),
-          "+r"(E[8]), "+r"(E[9]), "+r"(E[10]), "+r"(E[11]), "+r"(E[12]), "+r"(E[13])
-        : "r"(x0), "r"(b[0]), "r"(b[2]), "r"(b[4]), "r"(b[6]), "r"(b[8]), "r"(b[10]));
-    // O[0..11] += x0 b_odd, carry into O[12..13]
-    asm("mad.lo.cc.u32 %0, %14, %15, %0;\n\t"
-        "madc.hi.cc.u32 %1, %14, %15, %1;\n\t"
-        "madc.lo.cc.u32 %2, %14, %16, %2;\n\t"
-        "madc.hi.cc.u32 %3, %14, %16, %3;\n\t"
-        "madc.lo.cc.u32 %4, %14, %17, %4;\n\t"
-        "madc.hi.cc.u32 %5, %14, %17, %5;\n\t"
-        "madc.lo.cc.u32 %6, %14, %18, %6;\n\t"
-        "madc.hi.cc.u32 %7, %14, %18, %7;\n\t"
-        "madc.lo.cc.u32 %8, %14, %19, %8;\n\t"
-        "madc.hi.cc.u32 %9, %14, %19, %9;\n\t"
-        "madc.lo.cc.u32 %10, %14, %20, %10;\n\t"
-        "madc.hi.cc.u32 %11, %14, %20, %11;\n\t"
-        "addc.cc.u32 %12, %12, 0;\n\t"
-        "addc.u32 %13, %13, 0;"
-        : "+r"(O[0]), "+r"(O[1]), "+r"(O[2]), "+r"(O[3]), "+r"(O[4]), "+r"(O[5]), "+r"(O[6]), "+r"(O[7]),
-          "+r"(O[8]), "+r"(O[9]), "+r"(O[10]), "+r"(O[11]), "+r"(O[12]), "+r"(O[13])
-        : "r"(x0), "r"(b[1]), "r"(b[3]), "r"(b[5]), "r"(b[7]), "r"(b[9]), "r"(b[11]));
-    // O[0..11] += x1 b_even (limbs 1..12), carry into O[12..13]
-    asm("mad.lo.cc.u32 %0, %14, %15, %0;\n\t"
-        "madc.hi.cc.u32 %1, %14, %15, %1;\n\t"
-        "madc.lo.cc.u32 %2, %14, %16, %2;\n\t"
-        "madc.hi.cc.u32 %3, %14, %16, %3;\n\t"
-        "madc.lo.cc.u32 %4, %14, %17, %4;\n\t"
-        "madc.hi.cc.u32 %5, %14, %17, %5;\n\t"
-        "madc.lo.cc.u32 %6, %14, %18, %6;\n\t"
-        "madc.hi.cc.u32 %7, %14, %18, %7;\n\t"
-        "madc.lo.cc.u32 %8, %14, %19, %8;\n\t"
-        "madc.hi.cc.u32 %9, %14, %19, %9;\n\t"
-        "madc.lo.cc.u32 %10, %14, %20, %10;\n\t"
-        "madc.hi.cc.u32 %11, %14, %20, %11;\n\t"
-        "addc.cc.u32 %12, %12, 0;\n\t"
-        "addc.u32 %13, %13, 0;"
-        : "+r"(O[0]), "+r"(O[1]), "+r"(O[2]), "+r"(O[3]), "+r"(O[4]), "+r"(O[5]), "+r"(O[6]), "+r"(O[7]),
-          "+r"(O[8]), "+r"(O[9]), "+r"(O[10]), "+r"(O[11]), "+r"(O[12]), "+r"(O[13])
-        : "r"(x1), "r"(b[0]), "r"(b[2]), "r"(b[4]), "r"(b[6]), "r"(b[8]), "r"(b[10]));
-    // E[2..13] += x1 b_odd (limbs 2..13); no carry leaves E[13]
-    asm("mad.lo.cc.u32 %0, %12, %13, %0;\n\t"
-        "madc.hi.cc.u32 %1, %12, %13, %1;\n\t"
-        "madc.lo.cc.u32 %2, %12, %14, %2;\n\t"
-        "madc.hi.cc.u32 %3, %12, %14, %3;\n\t"
-        "madc.lo.cc.u32 %4, %12, %15, %4;\n\t"
-        "madc.hi.cc.u32 %5, %12, %15, %5;\n\t"
-        "madc.lo.cc.u32 %6, %12, %16, %6;\n\t"
-        "madc.hi.cc.u32 %7, %12, %16, %7;\n\t"
-        "madc.lo.cc.u32 %8, %12, %17, %8;\n\t"
-        "madc.hi.cc.u32 %9, %12, %17, %9;\n\t"
-        "madc.lo.cc.u32 %10, %12, %18, %10;\n\t"
-        "madc.hi.u32 %11, %12, %18, %11;"
-        : "+r"(E[2]), "+r"(E[3]), "+r"(E[4]), "+r"(E[5]), "+r"(E[6]), "+r"(E[7]), "+r"(E[8]), "+r"(E[9]),
-          "+r"(E[10]), "+r"(E[11]), "+r"(E[12]), "+r"(E[13])
-        : "r"(x1), "r"(b[1]), "r"(b[3]), "r"(b[5]), "r"(b[7]), "r"(b[9]), "r"(b[11]));
     const uint32_t m0 = (E[0] ^ neg1) + 1u;   // -E[0], through the opaque mask (neg_one)
     // O[0..11] += m0 p_odd (limbs 1..12), carry into O[12..13]
     asm("mad.lo.cc.u32 %0, %14, 0x8508c000, %0;\n\t"
@@ -409,6 +377,11 @@ __device__ __forceinline__ void mont_dstep(MontAccD& t, uint32_t x0, uint32_t x1
     O[12] = O[13] = 0;
 }
 
+__device__ __forceinline__ void mont_dstep(MontAccD& t, uint32_t x0, uint32_t x1, const uint32_t* b, uint32_t neg1) {
+    mont_rows(t, x0, x1, b);
+    mont_digits(t, neg1);
+}
+
 // r = E + 2^32 O after the last step (the words from 12 up cancel).
 __device__ __forceinline__ void mont_dfinal(fe& r, const MontAccD& t) {
     const uint32_t* e = t.e;
@@ -441,6 +414,24 @@ __device__ __forceinline__ void mul_inl(fe& r, const fe& a, const fe& b) {
     const uint32_t neg1 = neg_one();
 #pragma unroll
     for (int i = 0; i < N; i += 2) mont_dstep(t, a.v[i], a.v[i + 1], b.v, neg1);
+    mont_dfinal(r, t);
+}
+
+// r = (a1 b1 + a2 b2) R^-1 mod p in [0, 2p): one reduction for two products (420 instead
+// of 552 limb products). a1 b1 + a2 b2 < p R; within a step E stays below 2^445. (A
+// squaring with 78 instead of 144 products for the square itself was measured beside it:
+// right, but its shorter chains and its code cost what the products save: bucket
+// accumulation in XYZZ coordinates 5.56 -> 5.43 ms with it alone, 5.49 with both, 5.29 with
+// this alone.)
+__device__ __forceinline__ void mulsum_inl(fe& r, const fe& a1, const fe& b1, const fe& a2, const fe& b2) {
+    MontAccD t = {};
+    const uint32_t neg1 = neg_one();
+#pragma unroll
+    for (int i = 0; i < N; i += 2) {
+        mont_rows(t, a1.v[i], a1.v[i + 1], b1.v);
+        mont_rows(t, a2.v[i], a2.v[i + 1], b2.v);
+        mont_digits(t, neg1);
+    }
     mont_dfinal(r, t);
 }
 
@@ -493,6 +484,16 @@ __device__ __forceinline__ void mul2(fe& r1, const fe& a1, const fe& b1, fe& r2,
 }
 
 __device__ __forceinline__ void sqr(fe& r, const fe& a) { mul(r, a, a); }
+
+// r = (a1 b1 + a2 b2) R^-1 mod p.
+static __device__ __noinline__ fe mulsum_v(fe a1, fe b1, fe a2, fe b2) {
+    fe r;
+    mulsum_inl(r, a1, b1, a2, b2);
+    return r;
+}
+__device__ __forceinline__ void mulsum(fe& r, const fe& a1, const fe& b1, const fe& a2, const fe& b2) {
+    r = mulsum_v(a1, b1, a2, b2);
+}
 
 // r = a + b, inputs in [0, 2p); result folded into [0, 2p).
 __device__ __forceinline__ void add(fe& rr, const fe& a, const fe& bb) {
