@@ -216,9 +216,9 @@ __device__ __forceinline__ int unpack(const uint32_t* w, int lane) {
     return (int)(__funnelshift_r(lo, hi, sh) & (uint32_t)kDigit);
 }
 
-// The integer in limbs l[0..14] (|value| < 16 p) plus add0, as an element of [0, 2p)
-// on one thread: + 16 p, carries, packing, and one Montgomery product by R.
-__device__ __forceinline__ fq::fe to_fe(const int* l, int add0) {
+// c / R times (the integer in limbs l[0..14], |value| < 16 p, plus add0) mod p, in
+// [0, 2p), on one thread: + 16 p, carries, packing, and one Montgomery product by c.
+__device__ __forceinline__ fq::fe to_fe_times(const int* l, int add0, const fq::fe& c) {
     uint32_t w[13];
 #pragma unroll
     for (int k = 0; k < 13; ++k) w[k] = 0;
@@ -233,12 +233,18 @@ __device__ __forceinline__ fq::fe to_fe(const int* l, int add0) {
         w[i] |= (uint32_t)v;
         w[i + 1] |= (uint32_t)(v >> 32);
     }
-    fq::fe a, one;
+    fq::fe a;
 #pragma unroll
     for (int k = 0; k < 12; ++k) a.v[k] = w[k];
-    fq::set_one(one);
-    fq::mul(a, a, one);
+    fq::mul(a, a, c);
     return a;
+}
+
+// The integer itself mod p.
+__device__ __forceinline__ fq::fe to_fe(const int* l, int add0) {
+    fq::fe one;
+    fq::set_one(one);
+    return to_fe_times(l, add0, one);
 }
 
 // One thread: the limbs of a into slot i.
@@ -275,14 +281,15 @@ constexpr int kInvRounds = 33;
 
 // (a x + b y [+ m p]) / 2^27 per limb.
 template <bool kMod>
-__device__ __forceinline__ int shift_round(const Group& g, int a, int x, int b, int y) {
+__device__ __forceinline__ int shift_round(int lane, int p, int a, int x, int b, int y) {
     int64_t s = (int64_t)a * x + (int64_t)b * y;
-    if (kMod) s += (int64_t)(-from_lane(digit0(s), 0)) * g.p;
-    return from_lane(digit0(s), g.lane + 1) + digit1(s) + from_lane(digit2(s), g.lane + 31);
+    if (kMod) s += (int64_t)(-from_lane(digit0(s), 0)) * p;
+    return from_lane(digit0(s), lane + 1) + digit1(s) + from_lane(digit2(s), lane + 31);
 }
 
-__device__ __forceinline__ int inverse(const Group& g, const uint32_t* z) {
-    int f = g.p, gg = unpack(z, g.lane), d = 0, e = g.lane == 0 ? 1 : 0;
+// p: limb `lane` of p. Limb `lane` of the inverse (|value| < 16 p).
+__device__ __forceinline__ int inverse(int lane, int p, const uint32_t* z) {
+    int f = p, gg = unpack(z, lane), d = 0, e = lane == 0 ? 1 : 0;
     int delta2 = 1;                                    // 2 delta
     for (int round = 0; round < kInvRounds; ++round) {
         int fl = from_lane(f, 0), gl = from_lane(gg, 0);
@@ -302,8 +309,8 @@ __device__ __forceinline__ int inverse(const Group& g, const uint32_t* z) {
             u <<= 1;
             v <<= 1;
         }
-        const int f2 = shift_round<false>(g, u, f, v, gg), g2 = shift_round<false>(g, q, f, r, gg);
-        const int d2 = shift_round<true>(g, u, d, v, e), e2 = shift_round<true>(g, q, d, r, e);
+        const int f2 = shift_round<false>(lane, p, u, f, v, gg), g2 = shift_round<false>(lane, p, q, f, r, gg);
+        const int d2 = shift_round<true>(lane, p, u, d, v, e), e2 = shift_round<true>(lane, p, q, d, r, e);
         f = f2;
         gg = g2;
         d = d2;
@@ -311,6 +318,28 @@ __device__ __forceinline__ int inverse(const Group& g, const uint32_t* z) {
         if (!__any_sync(kFull, gg != 0)) break;
     }
     return digit0(from_lane(f, 0)) < 0 ? -d : d;       // f = +-1
+}
+
+// a^-1 of lane `src`'s a (Montgomery form, nonzero mod p) in every lane, on one warp; mem:
+// 28 words of shared memory of this warp's own.
+constexpr int kInverseWords = 28;
+__device__ __forceinline__ fq::fe inverse_fe(const fq::fe& a, int src, uint32_t* mem) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();                                      // earlier readers of mem are done
+    if (lane == src) {
+        fq::fe c;
+        fq::canon(c, a);
+        fq::store(mem, c);
+    }
+    __syncwarp();
+    const int v = inverse(lane, kP27[lane < 16 ? lane : 15], mem);   // (a R)^-1
+    int* limbs = reinterpret_cast<int*>(mem + 12);
+    if (lane < 16) limbs[lane] = v;
+    __syncwarp();
+    fq::fe r3;
+#pragma unroll
+    for (int k = 0; k < fq::N; ++k) r3.v[k] = fq::kR3[k];
+    return to_fe_times(limbs, 0, r3);                  // times R^2: a^-1 R
 }
 
 // ---------------------------------------------------------------- Edwards
@@ -440,7 +469,7 @@ struct Edwards {
         }
         __syncwarp();
         const bool ok = g.flags[0] == 0;               // warp-uniform
-        const int v = ok ? inverse(g, z) : 0;
+        const int v = ok ? inverse(g.lane, g.p, z) : 0;
         g.st(dst, v);
         return ok;
     }
