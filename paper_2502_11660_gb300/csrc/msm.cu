@@ -1119,10 +1119,11 @@ __global__ void k_bin_scatter(const uint32_t* __restrict__ kin, const uint32_t* 
 // holds items [t T, (t + 1) T); its block counts the tile's keys in 16-bit shared
 // counters packed two to a word (T < 2^16, so no count reaches the neighbour's
 // half) and gives each item its rank among the tile's items of the same key. The
-// tile counts go to cnt[w][t][key]; a column pass sums them into the bin totals, the
-// bin scan gives each (window, key) its offset, a second column pass turns cnt into
-// each tile's first slot per key (offset + counts of the earlier tiles), and an
-// item's slot is that plus its rank.
+// tile counts go to cnt[w][t][key]; a column pass (k_tile_totals) sums them into the bin
+// totals, scans these within blocks of bins and counts the pieces they will be cut into;
+// a second one (k_tile_offsets) adds the earlier blocks' totals, which gives each (window,
+// key) its offset, and turns cnt into each tile's first slot per key (offset + counts of
+// the earlier tiles); an item's slot is that plus its rank.
 constexpr int kTileThreads = 1024;
 constexpr uint32_t kTileItemsMax = 65535;
 constexpr size_t kTileSmemMax = 200 * 1024;    // packed counters of one block (GB300: 227 KB opt-in)
@@ -1154,40 +1155,6 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_count(const uint32_t* __r
     __syncthreads();
     uint32_t* cw = cnt + (w * ntiles + blockIdx.x) * nb;
     for (uint32_t k = threadIdx.x; k < nb; k += blockDim.x) cw[k] = (h[k >> 1] >> ((k & 1u) << 4)) & 0xffffu;
-}
-
-// Thread (w, key): bins[w][key] <- the count over the window's tiles.
-__global__ void k_tile_totals(const uint32_t* __restrict__ cnt, uint32_t nb, uint32_t ntiles, uint32_t W,
-                              uint32_t* __restrict__ bins) {
-    const size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (id >= (size_t)W * nb) return;
-    const size_t w = id / nb, k = id % nb;
-    const uint32_t* c = cnt + w * ntiles * nb + k;
-    uint32_t run = 0;
-    for (uint32_t t = 0; t < ntiles; ++t) run += c[(size_t)t * nb];
-    bins[id] = run;
-}
-
-// Thread (w, key), after the bin scan: cnt[w][t][key] <- the slot of the tile's first
-// item of that key, start[w][key] plus the counts of tiles t' < t.
-__global__ void k_tile_offsets(uint32_t* __restrict__ cnt, uint32_t nb, uint32_t ntiles, uint32_t W,
-                               const uint32_t* __restrict__ start) {
-    const size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (id >= (size_t)W * nb) return;
-    const size_t w = id / nb, k = id % nb;
-    uint32_t* c = cnt + w * ntiles * nb + k;
-    uint32_t run = start[id];
-    constexpr uint32_t kStep = 16;   // loads in flight per thread
-    for (uint32_t t0 = 0; t0 < ntiles; t0 += kStep) {
-        uint32_t v[kStep];
-#pragma unroll
-        for (uint32_t u = 0; u < kStep; ++u) v[u] = t0 + u < ntiles ? c[(size_t)(t0 + u) * nb] : 0u;
-#pragma unroll
-        for (uint32_t u = 0; u < kStep; ++u) {
-            if (t0 + u < ntiles) c[(size_t)(t0 + u) * nb] = run;
-            run += v[u];
-        }
-    }
 }
 
 // Grid (items of a window / 256, windows): each item to its tile's slot for the key
@@ -1265,19 +1232,104 @@ __device__ __forceinline__ BinRun bin_run(const PieceArgs& a, size_t id) {
     return r;
 }
 
+// The pieces of a run of m items, counted by length.
+__device__ __forceinline__ void count_pieces(uint32_t* h, uint32_t m, uint32_t cap) {
+    const uint32_t np = (m + cap - 1) / cap, q = m / np, big = m - q * np;
+    if (big) atomicAdd(&h[q + 1], big);
+    atomicAdd(&h[q], np - big);
+}
+
 __global__ void __launch_bounds__(kPieceThreads) k_piece_count(PieceArgs a) {
     __shared__ uint32_t h[kMaxPiece + 1];
     for (uint32_t k = threadIdx.x; k <= kMaxPiece; k += kPieceThreads) h[k] = 0;
     __syncthreads();
     const BinRun r = bin_run(a, blockIdx.x * (size_t)kPieceThreads + threadIdx.x);
-    if (r.m) {
-        const uint32_t np = (r.m + a.cap - 1) / a.cap, q = r.m / np, big = r.m - q * np;
-        if (big) atomicAdd(&h[q + 1], big);
-        atomicAdd(&h[q], np - big);
-    }
+    if (r.m) count_pieces(h, r.m, a.cap);
     __syncthreads();
     for (uint32_t k = threadIdx.x; k <= a.cap; k += kPieceThreads)
         if (h[k]) atomicAdd(&a.ctrl[kHist + k], h[k]);
+}
+
+// Counting sort by tiles, after k_tile_count. Thread (w, key): bins[w][key] <- the counts of
+// the block's earlier bins, bsum[block] <- the block's total, and the pieces of all bins
+// counted by length into hist (null: not counted here, several window groups). What bounds
+// these two kernels is the column reads (40 MB each way at n = 2^20, c = 16); small calls pay
+// their launches, and one launch each for totals, scan of the tiles, scan of the totals,
+// addition, piece counts and offsets was 10 to 15 us more than these two.
+constexpr int kBinBlock = 1024;
+
+__global__ void __launch_bounds__(kBinBlock) k_tile_totals(const uint32_t* __restrict__ cnt, uint32_t nb, uint32_t ntiles,
+                                                          uint32_t W, uint32_t* __restrict__ bins,
+                                                          uint32_t* __restrict__ bsum, uint32_t cap,
+                                                          uint32_t* __restrict__ hist) {
+    __shared__ uint32_t h[kMaxPiece + 1];
+    __shared__ uint32_t warp_tot[kBinBlock / 32];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    if (t <= (int)kMaxPiece) h[t] = 0;
+    __syncthreads();
+    const size_t id = blockIdx.x * (size_t)kBinBlock + t;
+    uint32_t m = 0;
+    if (id < (size_t)W * nb) {
+        const size_t w = id / nb, k = id - w * nb;
+        const uint32_t* c = cnt + w * ntiles * nb + k;
+        for (uint32_t u = 0; u < ntiles; ++u) m += c[(size_t)u * nb];
+        if (hist && k != 0 && m) count_pieces(h, m, cap);
+    }
+    uint32_t x = m;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_tot[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        uint32_t y = warp_tot[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t z = __shfl_up_sync(0xffffffffu, y, o);
+            if (lane >= o) y += z;
+        }
+        warp_tot[lane] = y;   // inclusive over warps
+    }
+    __syncthreads();
+    if (id < (size_t)W * nb) bins[id] = x - m + (wid ? warp_tot[wid - 1] : 0u);
+    if (t == kBinBlock - 1) bsum[blockIdx.x] = warp_tot[kBinBlock / 32 - 1];
+    if (hist && t <= (int)cap && h[t]) atomicAdd(&hist[t], h[t]);
+}
+
+// Thread (w, key): bins[w][key] <- the bin's offset, and cnt[w][t][key] <- the slot of tile
+// t's first item of that key, the offset plus the counts of tiles t' < t.
+__global__ void __launch_bounds__(256) k_tile_offsets(uint32_t* __restrict__ cnt, uint32_t nb, uint32_t ntiles, uint32_t W,
+                                                     uint32_t* __restrict__ bins, const uint32_t* __restrict__ bsum) {
+    __shared__ uint32_t part[8];
+    const int t = threadIdx.x;
+    const uint32_t block = blockIdx.x / (kBinBlock / 256);   // the block of bins that this one is in
+    uint32_t before = 0;
+    for (uint32_t b = t; b < block; b += 256) before += bsum[b];
+    before = __reduce_add_sync(0xffffffffu, before);
+    if ((t & 31) == 0) part[t >> 5] = before;
+    __syncthreads();
+    uint32_t run = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) run += part[k];
+    const size_t id = blockIdx.x * (size_t)256 + t;
+    if (id >= (size_t)W * nb) return;
+    const size_t w = id / nb, k = id - w * nb;
+    run += bins[id];
+    bins[id] = run;
+    uint32_t* c = cnt + w * ntiles * nb + k;
+    constexpr uint32_t kStep = 16;   // loads in flight per thread
+    for (uint32_t t0 = 0; t0 < ntiles; t0 += kStep) {
+        uint32_t v[kStep];
+#pragma unroll
+        for (uint32_t u = 0; u < kStep; ++u) v[u] = t0 + u < ntiles ? c[(size_t)(t0 + u) * nb] : 0u;
+#pragma unroll
+        for (uint32_t u = 0; u < kStep; ++u) {
+            if (t0 + u < ntiles) c[(size_t)(t0 + u) * nb] = run;
+            run += v[u];
+        }
+    }
 }
 
 // Appends the merge work of a bucket cut into np pieces; returns its first part slot.
@@ -1977,7 +2029,7 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool single = true) {
     p->off_dtot = take((size_t)p->W * (1u << p->rb) * 4);
     p->nbins = (size_t)p->W * (p->Bp + 1);  // keys 0 .. Bp of every window
     p->off_bins = take(p->nbins * 4);
-    p->off_bsum = take(((p->nbins + kScanTile - 1) / kScanTile) * 4);
+    p->off_bsum = take(((p->nbins + kBinBlock - 1) / kBinBlock) * 4);
     p->off_tcnt = take((size_t)p->W * p->ttiles * (p->Bp + 1) * 4);
     p->off_buckets = take((size_t)p->W * p->Bp * XY);
     p->off_parts = take(p->ngroups * p->max_parts * XY);
@@ -2223,6 +2275,7 @@ int enqueue_head(const Plan& p, const uint32_t* points, const uint32_t* scalars,
                                               p.sgn, p.user_bits, p.glv, keys[0], status);
     note_launches(1);
     int cur = 0;
+    bool pieces_counted = false;
     const int pre_w = p.pre ? p.Wd : 0;
     const uint32_t nb = p.Bp + 1;
     uint32_t* bins = at<uint32_t>(workspace, p.off_bins);
@@ -2231,7 +2284,6 @@ int enqueue_head(const Plan& p, const uint32_t* points, const uint32_t* scalars,
         const size_t total = (size_t)p.W * np;
         uint32_t* bsum = at<uint32_t>(workspace, p.off_bsum);
         uint32_t* rank = at<uint32_t>(workspace, p.off_rank);
-        const size_t ntiles = (p.nbins + kScanTile - 1) / kScanTile;
         const dim3 gw(grid_for(np, 256), (unsigned)p.W);
         uint32_t* tcnt = at<uint32_t>(workspace, p.off_tcnt);
         if (p.ttiles) {
@@ -2241,21 +2293,23 @@ int enqueue_head(const Plan& p, const uint32_t* points, const uint32_t* scalars,
                                               (int)kTileSmemMax));
             k_tile_count<<<dim3(p.ttiles, (unsigned)p.W), kTileThreads, smem, s>>>(keys[0], np, nb, p.tT, p.ttiles,
                                                                                   tcnt, rank);
-            k_tile_totals<<<grid_for(p.nbins, 256), 256, 0, s>>>(tcnt, nb, p.ttiles, (uint32_t)p.W, bins);
+            const PieceArgs a = piece_args(p, workspace, 0);
+            pieces_counted = p.ngroups == 1;
+            k_tile_totals<<<grid_for(p.nbins, kBinBlock), kBinBlock, 0, s>>>(
+                tcnt, nb, p.ttiles, (uint32_t)p.W, bins, bsum, a.cap, pieces_counted ? a.ctrl + kHist : nullptr);
+            k_tile_offsets<<<grid_for(p.nbins, 256), 256, 0, s>>>(tcnt, nb, p.ttiles, (uint32_t)p.W, bins, bsum);
+            k_tile_scatter<<<gw, 256, 0, s>>>(keys[0], rank, vals[0], total, np, nb, p.tT, p.ttiles, tcnt, p.np, pre_w);
+            note_launches(4);
         } else {
+            const size_t ntiles = (p.nbins + kScanTile - 1) / kScanTile;
             MSM_CUDA_TRY(cudaMemsetAsync(bins, 0, p.nbins * 4, s));
             k_bin_count<<<gw, 256, 0, s>>>(keys[0], np, nb, bins, rank);
-        }
-        k_scan_tiles<<<(unsigned)ntiles, kScanBlock, 0, s>>>(bins, p.nbins, bsum);
-        k_scan_totals<<<1, kScanBlock, 0, s>>>(bsum, ntiles);
-        k_scan_add<<<grid_for(p.nbins, 256), 256, 0, s>>>(bins, p.nbins, bsum);
-        if (p.ttiles) {
-            k_tile_offsets<<<grid_for(p.nbins, 256), 256, 0, s>>>(tcnt, nb, p.ttiles, (uint32_t)p.W, bins);
-            k_tile_scatter<<<gw, 256, 0, s>>>(keys[0], rank, vals[0], total, np, nb, p.tT, p.ttiles, tcnt, p.np, pre_w);
-        } else {
+            k_scan_tiles<<<(unsigned)ntiles, kScanBlock, 0, s>>>(bins, p.nbins, bsum);
+            k_scan_totals<<<1, kScanBlock, 0, s>>>(bsum, ntiles);
+            k_scan_add<<<grid_for(p.nbins, 256), 256, 0, s>>>(bins, p.nbins, bsum);
             k_bin_scatter<<<gw, 256, 0, s>>>(keys[0], rank, vals[0], total, np, nb, bins, p.np, pre_w);
+            note_launches(5);
         }
-        note_launches(p.ttiles ? 7 : 5);
     } else {
         uint32_t* hist = at<uint32_t>(workspace, p.off_hist);
         uint32_t* dtot = at<uint32_t>(workspace, p.off_dtot);
@@ -2278,9 +2332,12 @@ int enqueue_head(const Plan& p, const uint32_t* points, const uint32_t* scalars,
     for (int g = 0; g < p.ngroups; ++g) {
         const PieceArgs a = piece_args(p, workspace, g);
         const unsigned grid = grid_for((size_t)a.nwin * nb, kPieceThreads);
-        k_piece_count<<<grid, kPieceThreads, 0, s>>>(a);
+        if (!pieces_counted) {
+            k_piece_count<<<grid, kPieceThreads, 0, s>>>(a);
+            note_launches(1);
+        }
         k_piece_emit<<<grid, kPieceThreads, 0, s>>>(a);
-        note_launches(2);
+        note_launches(1);
     }
     return check_launch("msm head");
 }
