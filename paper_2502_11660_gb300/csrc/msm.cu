@@ -148,6 +148,7 @@ struct ModelXyzz {
     static __device__ __forceinline__ void add4_mem(acc& P, const uint4* q, fe* sh, int l) {
         ec::add4(P, MemQ{q}, sh, l, true);
     }
+    static __device__ __forceinline__ void exchange(acc& Q, const acc& P);   // the neighbour lane's point
     using chain = wred::Weierstrass;  // four-warp group operations (wred.cuh)
 };
 
@@ -199,6 +200,7 @@ struct ModelEdwards {
     static __device__ __forceinline__ void add4_mem(acc& P, const uint4* q, fe* sh, int l) {
         ed::add4(P, MemQE{q}, sh, l, true);
     }
+    static __device__ __forceinline__ void exchange(acc& Q, const acc& P);
     using chain = wred::Edwards;
 };
 
@@ -1656,6 +1658,57 @@ __global__ void __launch_bounds__(128) k_reduce_segments(const uint4* __restrict
     M::store(V + id * kXyzzVec, S);
 }
 
+__device__ __forceinline__ void shfl_xor_words(fe& r, const fe& a) {
+#pragma unroll
+    for (int k = 0; k < fq::N; ++k) r.v[k] = __shfl_xor_sync(0xffffffffu, a.v[k], 1);
+}
+
+__device__ __forceinline__ void ModelXyzz::exchange(acc& Q, const acc& P) {
+    shfl_xor_words(Q.X, P.X);
+    shfl_xor_words(Q.Y, P.Y);
+    shfl_xor_words(Q.ZZ, P.ZZ);
+    shfl_xor_words(Q.ZZZ, P.ZZZ);
+}
+__device__ __forceinline__ void ModelEdwards::exchange(acc& Q, const acc& P) {
+    shfl_xor_words(Q.X, P.X);
+    shfl_xor_words(Q.Y, P.Y);
+    shfl_xor_words(Q.Z, P.Z);
+    shfl_xor_words(Q.T, P.T);
+}
+
+// The same sums by two lanes per segment: the even lane runs T, the odd lane S one step
+// behind it, so a segment takes L additions in sequence instead of 2 (L - 1), and as many
+// threads serve half as many segments of twice the length: the bit sums that follow have
+// half the points. Measured, with the bit sums: 2^18 Edwards buckets 192 + 160 -> 222 + 106 us,
+// 17 windows of 2^14 XYZZ buckets 273 + 282 -> 307 + 175 us. At 2^19 XYZZ buckets the multiply
+// pipe bounds the one-thread form (580 us) and the estimate keeps it.
+template <class M>
+__global__ void __launch_bounds__(128) k_reduce_pairs(const uint4* __restrict__ buckets, uint32_t Bp, uint32_t L, int w0, int nwin,
+                               uint32_t G, uint4* __restrict__ Y, uint4* __restrict__ V) {
+    const size_t nseg = (size_t)nwin * G;
+    size_t id = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 1;
+    const bool run_s = threadIdx.x & 1, live = id < nseg;
+    if (!live) id = nseg - 1;   // whole warps go through the exchanges
+    const size_t wi = id / G, g = id % G;
+    const uint4* seg = buckets + ((size_t)(w0 + wi) * Bp + g * L) * kXyzzVec;
+    typename M::acc P, Q;
+    M::set_inf(P);
+    if (!run_s && !M::empty(seg + (size_t)(L - 1) * kXyzzVec)) M::load(P, seg + (size_t)(L - 1) * kXyzzVec);
+#pragma unroll 1
+    for (uint32_t i = 1; i <= L; ++i) {
+        M::exchange(Q, P);      // the odd lane adds T as it stands
+        if (!run_s) {           // the even lane the next bucket
+            M::set_inf(Q);
+            if (i < L) {
+                const uint4* b = seg + (size_t)(L - 1 - i) * kXyzzVec;
+                if (!M::empty(b)) M::load(Q, b);
+            }
+        }
+        M::add(P, Q);
+    }
+    if (live) M::store((run_s ? V : Y) + id * kXyzzVec, P);
+}
+
 // Sums of the segments' points by the bits of their index, four lanes per addition.
 // Per window there are (logG + 2) nb blocks: block (k, q), k < logG, sums the q-th of nb
 // equal slices of the G/2 points Y_g with bit k of g set (the j-th such index is j with
@@ -1785,6 +1838,7 @@ struct Plan {
     int ngroups;
     uint32_t L, G;
     uint32_t nb;     // blocks per bit of the segment sums
+    bool pairs;      // segments by two lanes each
     int logG, log2L;
     size_t off_status, off_ctrl, ctrl_bytes;   // status words, then the groups' counters: cleared together
     size_t off_points, off_keys0, off_vals0, off_keys1, off_vals1, off_rank, off_hist, off_dtot;
@@ -1982,6 +2036,9 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool single = true) {
             const size_t per_nb = (size_t)p->gw * (lg + 2);
             const double threads = (double)p->gw * G / (double)kWave;
             const double add1 = t1 > t1_full * threads ? t1 : t1_full * threads;
+            const double add2 = 1.1 * (t1 > 2 * t1_full * threads ? t1 : 2 * t1_full * threads);
+            const bool pairs = L >= 4 && L * add2 < 2.0 * (L - 1) * add1;
+            const double segments = L == 1 ? 0.0 : 3.0 + (pairs ? L * add2 : 2.0 * (L - 1) * add1);
             // a tuned number of segments: the longest L that leaves as many
             const bool forced = tr > 0;
             if (forced && L > 1 && (uint64_t)p->W * G < (1ull << tr)) break;
@@ -1991,7 +2048,7 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool single = true) {
                 const double in_blocks = blocks * kTreeWave * kTreeThreads / (double)kWave;
                 const uint32_t span = G / 2 / nb, by_thread = span > kTreeThreads ? span / kTreeThreads - 1 : 0;
                 const double steps = (double)((span < kTreeThreads ? span : kTreeThreads) + kTreeGroups - 1) / kTreeGroups + 4;
-                const double t = 2.0 * (L - 1) * add1 + (L > 1 ? 3.0 : 0.0) +
+                const double t = segments +
                                  by_thread * (t1 > t1_full * in_blocks ? t1 : t1_full * in_blocks) +
                                  steps * (t4 > t4_full * blocks ? t4 : t4_full * blocks) +
                                  (nb > 1 ? 3.0 + t4 * ilog2(nb) : 0.0);
@@ -1999,6 +2056,7 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool single = true) {
                     best = t;
                     p->L = L;
                     p->nb = nb;
+                    p->pairs = pairs;
                 }
             }
         }
@@ -2366,8 +2424,11 @@ int enqueue_group_tail_m(const Plan& p, const AccArgs& acc, int g, void* workspa
         const size_t yv = (size_t)p.gw * p.G * kXyzzVec;
         uint4* Y = at<uint4>(workspace, p.off_Y) + (size_t)g * yv;
         uint4* V = at<uint4>(workspace, p.off_V) + (size_t)g * yv;
-        k_reduce_segments<M><<<grid_for((size_t)a.nwin * p.G, 128), 128, 0, s>>>(a.buckets, p.Bp, p.L, a.w0, a.nwin, p.G,
-                                                                                Y, V);
+        const size_t nt = (size_t)a.nwin * p.G;
+        if (p.pairs)
+            k_reduce_pairs<M><<<grid_for(2 * nt, 128), 128, 0, s>>>(a.buckets, p.Bp, p.L, a.w0, a.nwin, p.G, Y, V);
+        else
+            k_reduce_segments<M><<<grid_for(nt, 128), 128, 0, s>>>(a.buckets, p.Bp, p.L, a.w0, a.nwin, p.G, Y, V);
         k_bit_sums<M, false><<<(unsigned)(nseg * p.nb), kTreeThreads, 0, s>>>(Y, V, a.nwin, p.G, p.logG, p.nb, P0);
         note_launches(2);
     } else {
