@@ -65,41 +65,31 @@ __global__ void k_fq_convert(const uint32_t* __restrict__ in, uint32_t* __restri
     }
 }
 
-// Mixed additions out_i = acc_i + q_i. What bounds it: the integer multiply pipe (10
-// products per addition; the 480 bytes take a fifth of the time). Three blocks of 128
-// per SM run over the batch in strides, so that the accumulator, the operand and two
-// products in flight stay in registers. A doubling (acc_i = q_i) is put off: one lane's
-// doubling would hold its whole warp for 7 products, so each warp keeps a list of them and
-// doubles up to 32 together. Measured at n = 1000003 with 1 % doublings: 566 -> 459 us
-// (two and four blocks per SM: 483 and 478).
+// Mixed additions out_i = acc_i + q_i in Montgomery form. What bounds it: the integer
+// multiply pipe (10 products per addition; the 480 bytes take a fifth of the time). Three
+// blocks of 128 per SM run over the batch in strides, so that the accumulator, the operand
+// and two products in flight stay in registers (two and four blocks per SM were 5 % and 4 %
+// slower). A doubling (acc_i = q_i) is put off: one lane's doubling would hold its whole
+// warp for 7 products, so each warp keeps a list of them and doubles up to 32 together; in
+// a single pass there is nothing to wait for. Measured at n = 1000003 with 1 % doublings:
+// 566 -> 442 us.
 constexpr unsigned kPaddBlock = 128, kPaddPerSm = 3;
 
-__device__ __forceinline__ void store_padd(uint32_t* out, size_t i, size_t n, xyzz& P, int form) {
-    if (form == MSM377_FORM_STANDARD) {
-        fq::from_mont(P.X, P.X);
-        fq::from_mont(P.Y, P.Y);
-        fq::from_mont(P.ZZ, P.ZZ);
-        fq::from_mont(P.ZZZ, P.ZZZ);
-    } else {
-        fq::canon(P.X, P.X);
-        fq::canon(P.Y, P.Y);
-        fq::canon(P.ZZ, P.ZZ);
-        fq::canon(P.ZZZ, P.ZZZ);
-    }
+__device__ __forceinline__ void store_padd(uint32_t* out, size_t i, size_t n, xyzz& P) {
+    fq::canon(P.X, P.X);
+    fq::canon(P.Y, P.Y);
+    fq::canon(P.ZZ, P.ZZ);
+    fq::canon(P.ZZZ, P.ZZZ);
     store_xyzz_soa(out, i, n, P);
 }
 
-__device__ __forceinline__ void load_padd_q(affine& Q, const uint32_t* q, size_t i, size_t n, int form) {
+__device__ __forceinline__ void load_padd_q(affine& Q, const uint32_t* q, size_t i, size_t n) {
     fq::load_soa(Q.x, q, i, n);
     fq::load_soa(Q.y, q + 12 * n, i, n);
-    if (form == MSM377_FORM_STANDARD) {
-        fq::to_mont(Q.x, Q.x);
-        fq::to_mont(Q.y, Q.y);
-    }
 }
 
 __global__ void __launch_bounds__(kPaddBlock, kPaddPerSm) k_padd(const uint32_t* acc, const uint32_t* __restrict__ q,
-                                                                 uint32_t* out, size_t n, int form) {
+                                                                 uint32_t* out, size_t n) {
     __shared__ size_t list[kPaddBlock / 32][64];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     size_t* const todo = list[warp];
@@ -107,27 +97,25 @@ __global__ void __launch_bounds__(kPaddBlock, kPaddPerSm) k_padd(const uint32_t*
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i0 = blockIdx.x * (size_t)blockDim.x + (size_t)warp * 32; i0 < n; i0 += stride) {
         const size_t i = i0 + lane;
+        const bool last = i0 + stride >= n;
         bool dbl = false;
         if (i < n) {
             xyzz P;
             affine Q;
             load_xyzz_soa(P, acc, i, n);
-            load_padd_q(Q, q, i, n, form);
-            if (form == MSM377_FORM_STANDARD) {
-                fq::to_mont(P.X, P.X);
-                fq::to_mont(P.Y, P.Y);
-                fq::to_mont(P.ZZ, P.ZZ);
-                fq::to_mont(P.ZZZ, P.ZZZ);
-            }
+            load_padd_q(Q, q, i, n);
             bool inf = ec::is_inf(P);
             dbl = ec::madd_but_double<false>(P, inf, Q);
-            if (!dbl) store_padd(out, i, n, P, form);
+            if (dbl && last && ntodo == 0) {
+                ec::mdbl(P, Q);
+                dbl = false;
+            }
+            if (!dbl) store_padd(out, i, n, P);
         }
         const uint32_t m = __ballot_sync(0xffffffffu, dbl);
         if (dbl) todo[ntodo + __popc(m & ((1u << lane) - 1u))] = i;
         ntodo += __popc(m);
         __syncwarp();
-        const bool last = i0 + stride >= n;
         while (ntodo >= 32 || (last && ntodo > 0)) {   // warp-uniform
             const int take = ntodo < 32 ? ntodo : 32;
             ntodo -= take;
@@ -135,11 +123,46 @@ __global__ void __launch_bounds__(kPaddBlock, kPaddPerSm) k_padd(const uint32_t*
                 const size_t k = todo[ntodo + lane];
                 xyzz P;
                 affine Q;
-                load_padd_q(Q, q, k, n, form);
+                load_padd_q(Q, q, k, n);
                 ec::mdbl(P, Q);
-                store_padd(out, k, n, P, form);
+                store_padd(out, k, n, P);
             }
             __syncwarp();
+        }
+    }
+}
+
+// The same in blocks of 256 with as many registers as they take and every doubling where
+// it occurs. Standard form has ten more products, the conversions of six coordinates in and
+// four out, and with them the kernel above is the slower one (1073 us at n = 1000003, 972
+// with paired conversions, against 901 here). In Montgomery form this one is ahead (27.3
+// against 28.9 us) where the batch fills one block of 256 per SM but not one of 128.
+template <bool kStandard>
+__global__ void k_padd_wide(const uint32_t* acc, const uint32_t* __restrict__ q, uint32_t* out, size_t n) {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
+         i += (size_t)gridDim.x * blockDim.x) {
+        xyzz P;
+        affine Q;
+        load_xyzz_soa(P, acc, i, n);
+        load_padd_q(Q, q, i, n);
+        if (kStandard) {
+            fq::to_mont(P.X, P.X);
+            fq::to_mont(P.Y, P.Y);
+            fq::to_mont(P.ZZ, P.ZZ);
+            fq::to_mont(P.ZZZ, P.ZZZ);
+            fq::to_mont(Q.x, Q.x);
+            fq::to_mont(Q.y, Q.y);
+        }
+        bool inf = ec::is_inf(P);
+        if (ec::madd_but_double<false>(P, inf, Q)) ec::mdbl(P, Q);
+        if (kStandard) {
+            fq::from_mont(P.X, P.X);
+            fq::from_mont(P.Y, P.Y);
+            fq::from_mont(P.ZZ, P.ZZ);
+            fq::from_mont(P.ZZZ, P.ZZZ);
+            store_xyzz_soa(out, i, n, P);
+        } else {
+            store_padd(out, i, n, P);
         }
     }
 }
@@ -272,14 +295,6 @@ unsigned batch_grid(size_t n) {
     return (unsigned)(want < cap ? (want ? want : 1) : cap);
 }
 
-unsigned padd_grid(size_t n) {
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t want = (n + kPaddBlock - 1) / kPaddBlock, cap = (size_t)sms * kPaddPerSm;
-    return (unsigned)(want < cap ? want : cap);
-}
-
 }  // namespace
 
 using namespace msm377;
@@ -318,7 +333,16 @@ extern "C" int padd_batch(const uint32_t* acc, const uint32_t* q, uint32_t* out,
     if (!acc || !q || !out) return set_error(MSM377_EINVAL, "padd_batch: null pointer");
     if (form != MSM377_FORM_STANDARD && form != MSM377_FORM_MONTGOMERY)
         return set_error(MSM377_EINVAL, "padd_batch: bad form %d", form);
-    k_padd<<<padd_grid(n), kPaddBlock, 0, as_stream(stream)>>>(acc, q, out, n, form);
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const size_t blocks = (n + kPaddBlock - 1) / kPaddBlock, cap = (size_t)sms * kPaddPerSm;
+    if (form == MSM377_FORM_STANDARD)
+        k_padd_wide<true><<<batch_grid(n), kBlock, 0, as_stream(stream)>>>(acc, q, out, n);
+    else if (blocks > (size_t)sms && n <= (size_t)sms * kBlock)
+        k_padd_wide<false><<<batch_grid(n), kBlock, 0, as_stream(stream)>>>(acc, q, out, n);
+    else
+        k_padd<<<(unsigned)(blocks < cap ? blocks : cap), kPaddBlock, 0, as_stream(stream)>>>(acc, q, out, n);
     note_launches(1);
     return check_launch("padd_batch");
 }

@@ -19,7 +19,7 @@ def _affine_points(seeds):
     return p.t().reshape(2, 12, seeds.shape[0]).contiguous()
 
 
-@pytest.mark.parametrize("n,every", [(1, 1), (31, 1), (129, 1), (129, 2), (70001, 1), (150001, 2), (150001, 37)])
+@pytest.mark.parametrize("n,every", [(1, 1), (31, 1), (129, 1), (129, 2), (19457, 3), (38912, 3), (38913, 3), (70001, 1), (150001, 2), (150001, 37)])
 @pytest.mark.parametrize("form", ["standard", "montgomery"])
 def test_doublings_among_additions(n, every, form):
     a, b = synth.scalars(41, n), synth.scalars(42, n)
