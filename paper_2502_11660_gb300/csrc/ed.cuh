@@ -103,17 +103,6 @@ __device__ __forceinline__ void madd(ext& P, const stored& Q) {
     fq::mul2(P.X, P.X, A, P.Y, B, P.Y);  // X3 = E F, Y3 = G H
 }
 
-// P += Q with an identity flag kept by the caller (the first point of a run is
-// a 1M assignment instead of a 7M addition).
-__device__ __forceinline__ void madd(ext& P, bool& p_inf, const stored& Q) {
-    if (p_inf) {
-        from_stored(P, Q);
-        p_inf = false;
-        return;
-    }
-    madd(P, Q);
-}
-
 // P += Q, both extended; Q's coordinates are fetched through `q` (a register or
 // memory loader with X/Y/Z/T accessors), so a Q in memory never occupies registers.
 // A = (Y1 - X1)(Y2 - X2), B = (Y1 + X1)(Y2 + X2), C = T1 k T2, D = 2 Z1 Z2, then as madd.
@@ -172,38 +161,11 @@ __device__ __forceinline__ void dbl(ext& P) {
     fq::mul2(P.Z, C, P.Y, P.Y, P.Y, A);  // F G, G H
 }
 
-// ---- four lanes per point operation (latency-bound chains; see ec::xchg4):
-// the multiplications of one Edwards formula fall into two or three levels of
-// independent products, so a doubling costs two multiplication latencies instead
-// of eight.
+// ---- four lanes per point operation (see ec::xchg4): the multiplications of one Edwards
+// formula fall into two or three levels of independent products, so an addition costs
+// three multiplication latencies instead of nine.
 using ec::pick4;
 using ec::xchg4;
-
-// P = 2P: level 1 {X^2, Y^2, Z^2, (X + Y)^2}, level 2 {E F, G H, E H, F G}.
-__device__ __forceinline__ void dbl4(ext& P, fe* sh, int l, bool writer) {
-    fe s, r, v[4];
-    fq::add_nr(s, P.X, P.Y);
-    const fe x = pick4(l, P.X, P.Y, P.Z, s);
-    fq::sqr(r, x);
-    xchg4(v, r, sh, l, writer);     // A, B, Z^2, (X + Y)^2
-    fe E, G, H, F, z;
-    fq::sub_nr<2>(E, v[3], v[0]);
-    fq::sub_nr<2>(E, E, v[1]);      // E = (X + Y)^2 - A - B
-    fq::sub_nr<2>(G, v[1], v[0]);   // G = B - A
-    fq::set_zero(z);
-    fq::sub_nr<2>(H, z, v[0]);
-    fq::sub_nr<2>(H, H, v[1]);      // H = -A - B
-    fq::add_nr(F, v[2], v[2]);
-    fq::sub_nr<4>(F, G, F);         // F = G - 2 Z^2 (ranges as in dbl)
-    const fe a = pick4(l, E, G, E, F);
-    const fe b = pick4(l, F, H, H, G);
-    fq::mul(r, a, b);
-    xchg4(v, r, sh, l, writer);     // X3, Y3, T3, Z3
-    P.X = v[0];
-    P.Y = v[1];
-    P.T = v[2];
-    P.Z = v[3];
-}
 
 // P += Q (extended, Q read through `q`): level 1 {A, B, T1 T2, Z1 Z2}, level 2
 // {k T1 T2} (one lane), level 3 {E F, G H, E H, F G}.

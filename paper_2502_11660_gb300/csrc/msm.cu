@@ -274,15 +274,54 @@ __device__ __forceinline__ fe shfl_fe_down(const fe& a, int off) {
     return r;
 }
 
+__device__ __forceinline__ fe shfl_fe(const fe& a, int src) {
+    fe r;
+#pragma unroll
+    for (int k = 0; k < fq::N; ++k) r.v[k] = __shfl_sync(0xffffffffu, a.v[k], src);
+    return r;
+}
+
 // The inverse of every lane's acc (nonzero on every lane) with one field inversion
 // for the warp: prefix products P_l = acc_0 ... acc_l and suffix products
 // S_l = acc_{l+1} ... acc_31 over the lanes give acc_l^-1 = total^-1 P_{l-1} S_l.
-// Every lane of the warp must call it; mem: wred::kInverseWords words of shared memory of
-// this warp's own. The one inversion runs on all lanes (wred::inverse) and the two scans
-// are paired: with a binary GCD on one lane, 80 us in which the others waited, and separate
-// scans, the preparation of 300007 GLV pairs took 389 us instead of 309, of 2^20 930 instead
-// of 857.
-__device__ __forceinline__ fe warp_lane_inverse(const fe& acc, uint32_t* mem) {
+// Every lane of the warp must call it. This form, a binary GCD on lane 0 and the two scans
+// one after the other, is the faster one in the fixed-base precomputation, whose doublings
+// keep the multiply pipe busy meanwhile (20000 points, c = 13: 9.5 ms, with the form below
+// 10.3).
+__device__ __forceinline__ fe warp_lane_inverse(const fe& acc) {
+    const int lane = threadIdx.x & 31;
+    fe one;
+    fq::set_one(one);
+    fe pre = acc, y;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {  // P_l
+        y = shfl_fe_up(pre, off);
+        if (lane >= off) fq::mul(pre, pre, y);
+    }
+    fe sacc = acc;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {  // acc_l ... acc_31
+        y = shfl_fe_down(sacc, off);
+        if (lane + off < 32) fq::mul(sacc, sacc, y);
+    }
+    fe suf = shfl_fe_down(sacc, 1);           // S_l
+    if (lane == 31) suf = one;
+    const fe total = shfl_fe(pre, 31);
+    fe tinv = one;
+    if (lane == 0) ec::inv(tinv, total);
+    tinv = shfl_fe(tinv, 0);
+    fe before = shfl_fe_up(pre, 1);           // P_{l-1}
+    if (lane == 0) before = one;
+    fe inv;
+    fq::mul(inv, tinv, before);
+    fq::mul(inv, inv, suf);
+    return inv;
+}
+
+// The same with the inversion on all lanes (wred::inverse) and the scans paired, for the
+// preparation, which waits for it: 300007 GLV pairs 389 -> 309 us, 2^20 930 -> 857. mem:
+// wred::kInverseWords words of shared memory of this warp's own.
+__device__ __forceinline__ fe warp_lane_inverse_wide(const fe& acc, uint32_t* mem) {
     const int lane = threadIdx.x & 31;
     fe one;
     fq::set_one(one);
@@ -311,7 +350,7 @@ __device__ __forceinline__ fe warp_lane_inverse(const fe& acc, uint32_t* mem) {
 // inverse of that product, from which it walks back through its chunk. Every lane
 // of the warp must call it (m may be 0; lanes carry 1 then).
 template <int K>
-__device__ __forceinline__ void warp_batch_inverse(fe (&den)[K], const bool (&ok)[K], int m, uint32_t* mem) {
+__device__ __forceinline__ void warp_batch_inverse(fe (&den)[K], const bool (&ok)[K], int m) {
     fe prefix[K];
     fe acc;
     fq::set_one(acc);
@@ -319,7 +358,7 @@ __device__ __forceinline__ void warp_batch_inverse(fe (&den)[K], const bool (&ok
         prefix[j] = acc;                   // product of the valid den[0..j-1]
         if (ok[j]) fq::mul(acc, acc, den[j]);
     }
-    fe inv = warp_lane_inverse(acc, mem);
+    fe inv = warp_lane_inverse(acc);
     for (int j = m - 1; j >= 0; --j) {
         if (!ok[j]) continue;
         fe dj;
@@ -348,7 +387,7 @@ __device__ __forceinline__ void store_ed_identity(uint4* o) {
 // an even start and end, so every lane's i0 and m are even.
 __device__ __forceinline__ void ed_affine_chunk(const uint4* __restrict__ in, size_t n, size_t np, size_t i0, int m,
                                                 bool pairs, fe (&xe)[kEdChunk], fe (&ye)[kEdChunk],
-                                                bool (&ok)[kEdChunk], uint32_t* mem) {
+                                                bool (&ok)[kEdChunk]) {
     fe one, sp;
     fq::set_one(one);
     ed::load_const(sp, ed::kS);
@@ -378,7 +417,7 @@ __device__ __forceinline__ void ed_affine_chunk(const uint4* __restrict__ in, si
             okv[3 * q + 1] = !id && !fq::is_zero(inv[3 * q + 1]);
             okv[3 * q + 2] = !id && !fq::is_zero(inv[3 * q + 2]);
         }
-        warp_batch_inverse(inv, okv, 3 * (m / 2), mem);
+        warp_batch_inverse(inv, okv, 3 * (m / 2));
         fe c1;
         ed::load_const(c1, ed::kC1);
         for (int q = 0; q < m / 2; ++q) {
@@ -407,7 +446,7 @@ __device__ __forceinline__ void ed_affine_chunk(const uint4* __restrict__ in, si
         fq::mul(den[j], ys[j], apl);
         ok[j] = ok[j] && !fq::is_zero(den[j]);
     }
-    warp_batch_inverse(den, ok, m, mem);
+    warp_batch_inverse(den, ok, m);
     for (int j = 0; j < m; ++j) {
         if (!ok[j]) continue;
         fe c, a;
@@ -487,7 +526,7 @@ constexpr int prep_blocks_per_sm(bool glv) { return glv ? 4 : 2; }
 //    y_e = (a - s) y / t.
 //  * A warp takes batches of 32 K consecutive points (lane l: points
 //    base + 32 q + l, q < K) and inverts all their t with one field inversion
-//    (Montgomery's trick over the lane's K points, warp_lane_inverse over the
+//    (Montgomery's trick over the lane's K points, warp_lane_inverse_wide over the
 //    lanes). Pass 1 writes each point's prefix product and the values pass 2
 //    needs into that point's own output rows; pass 2 reads them back (through
 //    L2) and overwrites the rows with the stored form.
@@ -534,7 +573,7 @@ __global__ void __launch_bounds__(128, prep_blocks_per_sm(kGlv))
             store_fe(o + 3, t);
             fq::mul(acc, acc, t);
         }
-        fe inv = warp_lane_inverse(acc, mem[threadIdx.x >> 5]);   // acc^-1 on every lane
+        fe inv = warp_lane_inverse_wide(acc, mem[threadIdx.x >> 5]);   // acc^-1 on every lane
         for (int q = K - 1; q >= 0; --q) {       // pass 2
             const size_t i = base + 32 * (size_t)q;
             if (i >= b) continue;
@@ -606,8 +645,6 @@ __global__ void __launch_bounds__(128, prep_blocks_per_sm(kGlv))
 // sum_j 2^(cj) sum_b b B_jb = sum_b b sum_j B'_jb with B' over the shifted points.
 __global__ void __launch_bounds__(128, 3) k_precompute_ed(const uint4* __restrict__ in, uint4* __restrict__ out,
                                                        size_t n, size_t np, int c, int Wd) {
-    __shared__ uint32_t all_mem[4][wred::kInverseWords];
-    uint32_t* const mem = all_mem[threadIdx.x >> 5];
     const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     const size_t i0 = t * kEdChunk;
     const int m = i0 >= np ? 0 : (int)(np - i0 < (size_t)kEdChunk ? np - i0 : (size_t)kEdChunk);
@@ -616,7 +653,7 @@ __global__ void __launch_bounds__(128, 3) k_precompute_ed(const uint4* __restric
     ed::ext P[kEdChunk];
     {
         fe xe[kEdChunk], ye[kEdChunk];
-        ed_affine_chunk(in, n, np, i0, m, np != n && (np & 1) == 0, xe, ye, ok, mem);  // rows [0, np): launch-wide
+        ed_affine_chunk(in, n, np, i0, m, np != n && (np & 1) == 0, xe, ye, ok);  // rows [0, np): launch-wide
         for (int q = 0; q < m; ++q) {
             uint4* o = out + (size_t)ModelEdwards::kStored * ((i0 + q) * (size_t)Wd);
             if (ok[q]) {
@@ -637,7 +674,7 @@ __global__ void __launch_bounds__(128, 3) k_precompute_ed(const uint4* __restric
             den[q] = P[q].Z;
             ok[q] = !fq::is_zero(P[q].Z);
         }
-        warp_batch_inverse(den, ok, m, mem);
+        warp_batch_inverse(den, ok, m);
         for (int q = 0; q < m; ++q) {
             uint4* o = out + (size_t)ModelEdwards::kStored * ((i0 + q) * (size_t)Wd + j);
             if (!ok[q]) {
