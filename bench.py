@@ -232,8 +232,8 @@ def op_counts(sc_host: np.ndarray, c: int, bits: int, edwards: bool, glv: bool, 
     stored = 144 if edwards else 96
     return {"windows": W, "madd": madds, "bucket_running_sum_adds": full_adds, "window_dbls": dbls,
             "products_per_madd": pm, "accumulate_products": madds * pm,
-            "accumulate_bytes": nonzero * (stored + 8),
-            "bytes_per_madd": f"{stored} B gathered stored point + 8 B sorted (key, value) pair"}
+            "accumulate_bytes": nonzero * (stored + 4),
+            "bytes_per_madd": f"{stored} B gathered stored point + 4 B sorted item"}
 
 
 # ---------------------------------------------------------------- clocks, traffic

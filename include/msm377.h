@@ -229,8 +229,8 @@ int msm_g1_set_window_table(const int32_t *c_by_log2n, int len, uint32_t flags);
 
 /* Installs one measured schedule entry for signed digits and n in [2^log2n, 2^(log2n+1))
  * in the table of the mode named by flags (MSM377_EDWARDS / MSM377_GLV /
- * MSM377_PRECOMPUTED): c (window width, used when opts.c == 0), chunk (items per
- * accumulation thread, 2..256), sort (1 counting sort, 2 LSD radix sort),
+ * MSM377_PRECOMPUTED): c (window width, used when opts.c == 0), chunk (items of
+ * the longest piece an accumulation thread sums, 2..256), sort (1 counting sort, 2 LSD radix sort),
  * reduce_log2 (log2 of the level-1 bucket-reduction threads, 8..20) and groups
  * (window groups, 1..8: the accumulation runs group by group and each group's
  * merges and bucket reduction run on a high-priority helper stream of the caller's
@@ -358,7 +358,7 @@ int msm_g1_resident_host(msm_points_t handle, size_t offset, size_t n, const uin
  * Batched MSM: many independent MSMs of uneven size in one call. The per-job
  * preparation, digits and sort run on library-owned helper streams; the bucket
  * accumulation of all jobs is one persistent kernel that drains a queue of
- * (job, window, chunk) items; the jobs' reductions and window combinations run
+ * the jobs' pieces; the jobs' reductions and window combinations run
  * on the helper streams again, so the serial tails overlap each other. Every
  * step forks from and joins back into opts->stream through events, so the call
  * can be captured into a CUDA graph once the first call on the device has
@@ -389,8 +389,8 @@ int msm_g1_status(const void *workspace, const msm_opts *opts);
 /* End-to-end variant on host buffers (synchronous): copies points_host (24 u32
  * per point, standard form) and scalars_host (8 u32 per scalar) into the
  * workspace, runs the MSM and copies the 24-u32 result into out_host. The points
- * travel in 2 chunks on a library helper stream and each chunk is prepared (the
- * options' curve model / GLV form) on a second helper stream as soon as it has
+ * travel in 4 chunks on a library helper stream and each chunk is prepared (the
+ * options' curve model / GLV form) on a helper stream of its own as soon as it has
  * arrived, while the scalars' copy, digits and bucket sort run on opts->stream;
  * the accumulation starts when the last chunk is prepared. Host buffers may be
  * pageable; pinned buffers copy faster and overlap. workspace (device, 256-byte

@@ -466,7 +466,7 @@ def msm_g1_set_schedule(log2n: int, c: int = 0, chunk: int = 0, sort: int = 0, r
 
 def msm_g1_schedule(n: int, c: int = 0, signed: bool = True, scalar_bits: int = 0, prepared: bool = True,
                     edwards: bool = False, glv: bool = False, precomputed: bool = False) -> dict:
-    """The schedule msm_g1 uses for these options: window c, chunk K, sort, level-1 reduction threads."""
+    """The schedule msm_g1 uses for these options: window c, longest piece K (chunk), sort, level-1 reduction threads."""
     o = _opts(c, signed, scalar_bits, prepared or precomputed, edwards=edwards, glv=glv, precomputed=precomputed)
     out = (ctypes.c_int32 * 5)()
     check(lib().msm_g1_schedule(n, ctypes.byref(o), out))

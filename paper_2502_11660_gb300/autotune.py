@@ -9,7 +9,7 @@ Tables can be saved to and loaded from a JSON file keyed by the device name.
 
 One synthetic point set of the largest size tuned is generated on the device and
 prepared once per curve model; smaller sizes time a prefix of it. tune_schedule()
-also searches, per size, the accumulation chunk size, the sort and the bucket
+also searches, per size, the longest accumulation piece ("chunk"), the sort and the bucket
 reduction's parallelism (msm_g1_set_schedule), one coordinate at a time.
 """
 from __future__ import annotations
@@ -134,7 +134,7 @@ def time_schedule(n: int, c: int, chunk: int, sort: int, reduce_log2: int, group
     return time_msm(n, 0, reps, device, seed, edwards=edwards, glv=glv)
 
 
-# chunk sizes (items per accumulation thread), sorts (1 counting, 2 radix), level-1
+# chunk (items of the longest accumulation piece), sorts (1 counting, 2 radix), level-1
 # reduction thread counts and window groups searched after the window width
 CHUNKS = (0, 16, 32, 48, 64, 96, 128)
 SORTS = (1, 2)

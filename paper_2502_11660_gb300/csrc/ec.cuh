@@ -225,9 +225,9 @@ __device__ __forceinline__ void add(xyzz& P, const xyzz& Q) { add_q(P, RegQ{&Q})
 
 // ---- four lanes per point operation (latency-bound chains)
 //
-// A dependent chain of point operations (the window combination, the per-window
-// Horner sums) runs at the latency of one thread's multiplications. The
-// multiplications inside one formula fall into a few levels of independent
+// A dependent chain of point operations (the trees that put the parts of cut buckets
+// together, the bit sums of the bucket reduction) runs at the latency of one thread's
+// multiplications. Those inside one formula fall into a few levels of independent
 // products, so four lanes of a warp that hold the same point each compute one
 // product of a level and exchange the results through shared memory. Every lane
 // of the warp calls these functions (lanes of the same group of four hold the same

@@ -507,8 +507,8 @@ __device__ __forceinline__ fe mont_one() {
 }
 
 // Blocks of 128 per SM for the Edwards preparation: the GLV form at four (128
-// registers, a few spills), the single-row form at two (its measured best: 0.54 ms for
-// 2^20 points against 0.60 at four).
+// registers, a few spills), the single-row form at two (its measured best, 0.485 ms for
+// 2^20 points).
 constexpr int prep_blocks_per_sm(bool glv) { return glv ? 4 : 2; }
 
 // Stored Edwards rows of input points [a, b): row i, or rows 2i and 2i + 1 (P_i and
@@ -1041,7 +1041,7 @@ __global__ void k_run_starts(const uint32_t* __restrict__ keys, size_t n, uint32
 // bin offsets (window w's bins start at w np, since each window holds np items),
 // and one pass scatters every item to its bin's next free slot. The order inside
 // a bin is not kept -- it does not matter, since a bucket's sum is the same group
-// element in any order. Two passes over the (key, value) pairs instead of a
+// element in any order. Two passes over the keys instead of a
 // histogram and a scatter pass per 8 key bits.
 constexpr int kScanBlock = 1024, kScanPer = 4, kScanTile = kScanBlock * kScanPer;
 
@@ -1899,7 +1899,7 @@ int ilog2(uint64_t v) {
 // GLV, fixed-base), set from measured tables by msm_g1_set_window_table (window
 // widths) and msm_g1_set_schedule (every field); 0 = the built-in rule.
 std::atomic<int> g_ctable[8][32];      // window width c
-std::atomic<int> g_ktable[8][32];      // items per accumulation chunk K
+std::atomic<int> g_ktable[8][32];      // longest piece K
 std::atomic<int> g_sorttable[8][32];   // 1 counting sort, 2 LSD radix sort
 std::atomic<int> g_rtable[8][32];      // log2 of the level-1 reduction threads
 std::atomic<int> g_gtable[8][32];      // window groups (1 = no overlap of tails with accumulation)
