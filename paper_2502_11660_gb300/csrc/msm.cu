@@ -31,6 +31,7 @@
 // windows (subgroup points); stored rows 2i and 2i + 1 are P_i and phi(P_i).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 
@@ -2027,7 +2028,7 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool single = true, size_t 
     // standard deviations, so that with at least a wave of buckets only unusually long
     // runs are cut (random digits leave hardly any); up to a third of a resident thread's
     // share of all items, so that a piece never outlasts the rest of the work, and up
-    // to two shares, so that every resident thread (152 SMs x kAccBlocks blocks of 128 on
+    // to one or two shares, so that every resident thread (152 SMs x kAccBlocks blocks of 128 on
     // a GB300) has work where buckets are few.
     const size_t kWave = (size_t)152 * 128 * (p->edw ? ModelEdwards::kAccBlocks : ModelXyzz::kAccBlocks);
     const size_t total = (size_t)p->gw * items;
@@ -2041,7 +2042,13 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool single = true, size_t 
     // longer than 48 on that account, as the queue's last job would end late (30 jobs of
     // 2^10 to 2^13 points 2.65 -> 2.19 ms; 24 of 2^10 to 2^18 7.17 -> 6.94, without the 48 7.24).
     const size_t shared = batch_items / kWave / 2 < 48 ? batch_items / kWave / 2 : 48;
-    const size_t longest = 2 * share + 4 > shared ? 2 * share + 4 : shared;
+    // Long shares: little more than one, or runs shorter than expected (zero digits) stay
+    // whole and leave threads idle where buckets are fewer than threads; short shares: two,
+    // as the parts' merges cost more there. Against two shares throughout, c = 12, XYZZ:
+    // 262144 GLV pairs, half the digits zero, 2819 -> 1845 us; 262144 points 3411 -> 2720 us. One
+    // share throughout: 30071 GLV pairs, c = 9, 960 -> 1426 us.
+    const size_t two = 2 * share + 4, most = batch_items ? two : std::max(share + 4, std::min<size_t>(two, 36));
+    const size_t longest = most > shared ? most : shared;
     if (K > longest) K = longest;
     if (K < 2) K = 2;
     if (K > kMaxPiece) K = kMaxPiece;
