@@ -694,11 +694,12 @@ __global__ void __launch_bounds__(128, 3) k_precompute_ed(const uint4* __restric
 
 // Window digits of one scalar (8 words, little-endian) for point index `idx`:
 // |digit| (0 = no contribution) with its sign in bit 31, window-major ([W][np]). The
-// point of an item follows from its place (item_point), so it is not stored.
-__device__ __forceinline__ void emit_digits(const uint32_t (&s)[8], int c, int W, int sgn, size_t idx,
+// point of an item follows from its place (item_point), so it is not stored. Returns how
+// many digits are not zero.
+__device__ __forceinline__ uint32_t emit_digits(const uint32_t (&s)[8], int c, int W, int sgn, size_t idx,
                                             size_t np, uint32_t* __restrict__ keys) {
     const uint32_t cmask = (1u << c) - 1u, half = 1u << (c - 1);
-    uint32_t carry = 0;
+    uint32_t carry = 0, nonzero = 0;
     for (int j = 0; j < W; ++j) {
         int b0 = j * c, w = b0 >> 5, off = b0 & 31;
         uint32_t raw = 0;
@@ -722,7 +723,9 @@ __device__ __forceinline__ void emit_digits(const uint32_t (&s)[8], int c, int W
             key = raw;
         }
         keys[(size_t)j * np + idx] = key | (neg << 31);
+        nonzero += key != 0;
     }
+    return nonzero;
 }
 
 constexpr uint32_t kSign = 0x80000000u;
@@ -839,10 +842,9 @@ __device__ __forceinline__ void glv_split(uint32_t (&k)[8], uint32_t (&k1)[8], u
     }
 }
 
-__global__ void k_digits(const uint4* __restrict__ scalars, size_t n, int c, int W, int sgn,
-                         int bits, int glv, uint32_t* __restrict__ keys, int* __restrict__ status) {
-    size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
+// The digits of scalar i; returns how many are not zero.
+__device__ __forceinline__ uint32_t scalar_digits(const uint4* __restrict__ scalars, size_t i, size_t n, int c, int W, int sgn,
+                                                  int bits, int glv, uint32_t* __restrict__ keys, int* __restrict__ status) {
     uint4 lo = scalars[2 * i], hi = scalars[2 * i + 1];
     uint32_t s[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
     if (bits < 256) {
@@ -856,14 +858,30 @@ __global__ void k_digits(const uint4* __restrict__ scalars, size_t n, int c, int
         }
         if (over) atomicCAS(status, 0, MSM377_ERANGE);   // the first error of the call stays
     }
-    if (!glv) {
-        emit_digits(s, c, W, sgn, i, n, keys);
-        return;
-    }
+    if (!glv) return emit_digits(s, c, W, sgn, i, n, keys);
     uint32_t k1[8], k2[8];
     glv_split(s, k1, k2);
-    emit_digits(k1, c, W, sgn, 2 * i, 2 * n, keys);      // P_i
-    emit_digits(k2, c, W, sgn, 2 * i + 1, 2 * n, keys);  // phi(P_i)
+    const uint32_t m = emit_digits(k1, c, W, sgn, 2 * i, 2 * n, keys);     // P_i
+    return m + emit_digits(k2, c, W, sgn, 2 * i + 1, 2 * n, keys);         // phi(P_i)
+}
+
+// nonzero: the count of digits that are not zero is added there (null: not counted; see
+// piece_cap).
+constexpr int kDigitThreads = 256;
+
+__global__ void __launch_bounds__(kDigitThreads) k_digits(const uint4* __restrict__ scalars, size_t n, int c, int W, int sgn,
+                                                          int bits, int glv, uint32_t* __restrict__ keys,
+                                                          int* __restrict__ status, uint32_t* __restrict__ nonzero) {
+    __shared__ uint32_t block_count;
+    if (threadIdx.x == 0) block_count = 0;
+    const size_t i = blockIdx.x * (size_t)kDigitThreads + threadIdx.x;
+    uint32_t m = i < n ? scalar_digits(scalars, i, n, c, W, sgn, bits, glv, keys, status) : 0u;
+    if (!nonzero) return;   // the whole grid
+    __syncthreads();
+    m = __reduce_add_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&block_count, m);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(nonzero, block_count);
 }
 
 // ---------------------------------------------------------------- stage 3: radix sort
@@ -1260,14 +1278,22 @@ constexpr int kPieceThreads = 256;
 
 // Device counters of one window group, zeroed before use. Indices into uint32_t words.
 enum : uint32_t { kHist = 0, kCursor = kMaxPiece + 1, kNParts = 2 * (kMaxPiece + 1), kNSmall, kNTree /* 3 levels */,
-                  kCtrlWords = (kNTree + 3 + 31) / 32 * 32 };
+                  kNonzero = kNTree + 3 /* the first group's: digits of all groups */,
+                  kCtrlWords = (kNonzero + 1 + 31) / 32 * 32 };
 
 struct PieceArgs {
     const uint32_t* start;  // first item of each bin (w, key), key < nb; the next bin's start ends it
     uint32_t nb, Bp;
     int w0, nwin;           // windows of this group
     uint32_t total;         // all windows' items: the end of the last bin
-    uint32_t cap;
+    uint32_t cap;           // longest piece where most digits are nonzero (piece_cap)
+    uint32_t cap_few;       // and the shortest that it may become where few are
+    const uint32_t* nonzero;   // digits that are not zero, over all windows (null: cap as it is)
+    uint32_t all;           // items of all windows
+    uint32_t group_items;   // items of a full group
+    uint32_t wave;          // resident threads
+    uint32_t shared;        // half a thread's share of the whole batch's items (0: a single call)
+    int levels;             // tree levels of the merge that are launched
     uint32_t small_parts;   // buckets of up to this many parts are summed by one thread
     uint32_t* ctrl;
     uint4* pieces;          // {first item, length, destination, -}
@@ -1296,6 +1322,25 @@ __device__ __forceinline__ BinRun bin_run(const PieceArgs& a, size_t id) {
     return r;
 }
 
+// The longest piece. cap takes every digit for nonzero, but a thread's share is of those
+// that are: 2^20 scalars of one, c = 12, Edwards + GLV, are one run of 2^20 points among 23
+// million zero digits, and in pieces of cap = 256 it kept 4096 threads for 1925 us. With
+// fewer than half the digits nonzero the piece is a thread's share of them (plus 4, as in
+// make_plan), but no shorter than cap_few, nor so short that the pieces of the nonzero digits
+// outgrow the bound group_items / cap on which the lists are sized.
+__device__ __forceinline__ uint32_t piece_cap(const PieceArgs& a) {
+    if (!a.nonzero) return a.cap;
+    const uint32_t nz = *a.nonzero;
+    if (nz >= a.all / 2) return a.cap;
+    const uint32_t bound = (uint32_t)(((uint64_t)nz * a.cap + a.group_items - 1) / a.group_items);
+    uint32_t k = nz / a.wave + 5;
+    const uint32_t shared = (uint32_t)((uint64_t)nz * a.shared / a.all);
+    if (k < shared) k = shared;
+    if (k < bound) k = bound;
+    if (k < a.cap_few) k = a.cap_few;
+    return k < a.cap ? k : a.cap;
+}
+
 // The pieces of a run of m items, counted by length.
 __device__ __forceinline__ void count_pieces(uint32_t* h, uint32_t m, uint32_t cap) {
     const uint32_t np = (m + cap - 1) / cap, q = m / np, big = m - q * np;
@@ -1308,7 +1353,7 @@ __global__ void __launch_bounds__(kPieceThreads) k_piece_count(PieceArgs a) {
     for (uint32_t k = threadIdx.x; k <= kMaxPiece; k += kPieceThreads) h[k] = 0;
     __syncthreads();
     const BinRun r = bin_run(a, blockIdx.x * (size_t)kPieceThreads + threadIdx.x);
-    if (r.m) count_pieces(h, r.m, a.cap);
+    if (r.m) count_pieces(h, r.m, piece_cap(a));
     __syncthreads();
     for (uint32_t k = threadIdx.x; k <= a.cap; k += kPieceThreads)
         if (h[k]) atomicAdd(&a.ctrl[kHist + k], h[k]);
@@ -1316,7 +1361,7 @@ __global__ void __launch_bounds__(kPieceThreads) k_piece_count(PieceArgs a) {
 
 // Counting sort by tiles, after k_tile_count. Thread (w, key): bins[w][key] <- the counts of
 // the block's earlier bins, bsum[block] <- the block's total, and the pieces of all bins
-// counted by length into hist (null: not counted here, several window groups). What bounds
+// counted by length (pieces = 0: not counted here, several window groups). What bounds
 // these two kernels is the column reads (40 MB each way at n = 2^20, c = 16); small calls pay
 // their launches, and one launch each for totals, scan of the tiles, scan of the totals,
 // addition, piece counts and offsets was 10 to 15 us more than these two.
@@ -1324,8 +1369,7 @@ constexpr int kBinBlock = 1024;
 
 __global__ void __launch_bounds__(kBinBlock) k_tile_totals(const uint32_t* __restrict__ cnt, uint32_t nb, uint32_t ntiles,
                                                           uint32_t W, uint32_t* __restrict__ bins,
-                                                          uint32_t* __restrict__ bsum, uint32_t cap,
-                                                          uint32_t* __restrict__ hist) {
+                                                          uint32_t* __restrict__ bsum, PieceArgs a, int pieces) {
     __shared__ uint32_t h[kMaxPiece + 1];
     __shared__ uint32_t warp_tot[kBinBlock / 32];
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
@@ -1337,7 +1381,7 @@ __global__ void __launch_bounds__(kBinBlock) k_tile_totals(const uint32_t* __res
         const size_t w = id / nb, k = id - w * nb;
         const uint32_t* c = cnt + w * ntiles * nb + k;
         for (uint32_t u = 0; u < ntiles; ++u) m += c[(size_t)u * nb];
-        if (hist && k != 0 && m) count_pieces(h, m, cap);
+        if (pieces && k != 0 && m) count_pieces(h, m, piece_cap(a));
     }
     uint32_t x = m;
 #pragma unroll
@@ -1359,7 +1403,7 @@ __global__ void __launch_bounds__(kBinBlock) k_tile_totals(const uint32_t* __res
     __syncthreads();
     if (id < (size_t)W * nb) bins[id] = x - m + (wid ? warp_tot[wid - 1] : 0u);
     if (t == kBinBlock - 1) bsum[blockIdx.x] = warp_tot[kBinBlock / 32 - 1];
-    if (hist && t <= (int)cap && h[t]) atomicAdd(&hist[t], h[t]);
+    if (pieces && t <= (int)a.cap && h[t]) atomicAdd(&a.ctrl[kHist + t], h[t]);
 }
 
 // Thread (w, key): bins[w][key] <- the bin's offset, and cnt[w][t][key] <- the slot of tile
@@ -1398,16 +1442,17 @@ __global__ void __launch_bounds__(256) k_tile_offsets(uint32_t* __restrict__ cnt
 
 // Appends the merge work of a bucket cut into np pieces; returns its first part slot.
 __device__ __forceinline__ uint32_t plan_merge(const PieceArgs& a, uint32_t np, uint32_t bucket) {
+    // partial sums of the tree's inner levels; the last level launched takes what is left
     const uint32_t n1 = (np + kTreeParts - 1) / kTreeParts, n2 = (n1 + kTreeParts - 1) / kTreeParts;
-    const uint32_t extra = np <= a.small_parts || n1 == 1 ? 0 : (n2 == 1 ? n1 : n1 + n2);
+    const uint32_t extra = np <= a.small_parts || n1 == 1 || a.levels == 1 ? 0 : (n2 == 1 || a.levels == 2 ? n1 : n1 + n2);
     const uint32_t base = atomicAdd(&a.ctrl[kNParts], np + extra);
     if (np <= a.small_parts) {
         a.small[atomicAdd(&a.ctrl[kNSmall], 1u)] = make_uint4(base, np, bucket, 0u);
         return base;
     }
     uint32_t src = base, cnt = np;
-    for (int lv = 0; lv < 3; ++lv) {
-        const uint32_t nout = lv == 2 ? 1u : (cnt + kTreeParts - 1) / kTreeParts;
+    for (int lv = 0; lv < a.levels; ++lv) {
+        const uint32_t nout = lv + 1 == a.levels ? 1u : (cnt + kTreeParts - 1) / kTreeParts;
         const uint32_t e = atomicAdd(&a.ctrl[kNTree + lv], nout);
         if (nout == 1) {
             a.tree[lv][e] = make_uint4(src, cnt, bucket, 0u);
@@ -1446,7 +1491,8 @@ __global__ void __launch_bounds__(kPieceThreads) k_piece_emit(PieceArgs a) {
     const BinRun r = bin_run(a, id);
     uint32_t np = 0, q = 0, big = 0, rank_big = 0, rank_q = 0;
     if (r.m) {
-        np = (r.m + a.cap - 1) / a.cap;
+        const uint32_t cap = piece_cap(a);
+        np = (r.m + cap - 1) / cap;
         q = r.m / np;
         big = r.m - q * np;
         if (big) rank_big = atomicAdd(&h[q + 1], big);
@@ -1894,6 +1940,10 @@ struct Plan {
     int passes, rb;  // radix-sort passes of rb-bit digits
     size_t tiles;
     int K;          // longest piece of a bucket's run
+    int K_few;      // and where few digits are nonzero, at least (piece_cap)
+    size_t shared;  // half a thread's share of the batch (0: a single call)
+    int levels;     // tree levels of the merge
+    size_t wave;    // resident accumulation threads
     uint32_t small_parts;   // parts that one thread puts together
     size_t max_pieces, max_parts, max_small, max_tree[3];   // per group: bounds over any digits
     int gw;         // windows per group
@@ -2073,11 +2123,21 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool single = true, size_t 
     // share throughout: 30071 GLV pairs, c = 9, 960 -> 1426 us.
     const size_t two = 2 * share + 4, most = batch_items ? two : std::max(share + 4, std::min<size_t>(two, 36));
     const size_t longest = most > shared ? most : shared;
+    // where few digits are nonzero: no shorter than the merges are worth, nor, in a batch, than
+    // for the job alone
+    const size_t few = batch_items ? two : 36;
     if (K > longest) K = longest;
     if (K < 2) K = 2;
     if (K > kMaxPiece) K = kMaxPiece;
     if (tk > 0) K = (size_t)tk;        // measured choice (2..256)
     p->K = (int)K;
+    p->K_few = tk > 0 || K < few ? (int)K : (int)few;
+    p->shared = batch_items / kWave / 2;
+    p->wave = kWave;
+    {
+        const size_t parts = (items + K - 1) / K;   // of one bucket, all digits nonzero
+        p->levels = parts > (size_t)kTreeParts * kTreeParts ? 3 : parts > kTreeParts ? 2 : items > (size_t)p->K_few ? 1 : 0;
+    }
     {
         // sum over buckets of ceil(m / K): at most one piece more than m / K per bucket in
         // use; a bucket with parts has more than K items
@@ -2362,6 +2422,13 @@ PieceArgs piece_args(const Plan& p, void* workspace, int g) {
     a.nwin = p.W - a.w0 < p.gw ? p.W - a.w0 : p.gw;
     a.total = (uint32_t)((size_t)(a.w0 + a.nwin) * p.items);
     a.cap = (uint32_t)p.K;
+    a.cap_few = (uint32_t)p.K_few;
+    a.nonzero = p.K_few < p.K ? at<uint32_t>(workspace, p.off_ctrl) + kNonzero : nullptr;
+    a.all = (uint32_t)((size_t)p.W * p.items);
+    a.group_items = (uint32_t)((size_t)p.gw * p.items);
+    a.wave = (uint32_t)p.wave;
+    a.shared = (uint32_t)p.shared;
+    a.levels = p.levels;
     a.small_parts = p.small_parts;
     a.ctrl = at<uint32_t>(workspace, p.off_ctrl) + (size_t)g * kCtrlWords;
     a.pieces = at<uint4>(workspace, p.off_pieces) + (size_t)g * p.max_pieces;
@@ -2404,8 +2471,10 @@ int enqueue_head(const Plan& p, const uint32_t* points, const uint32_t* scalars,
     const size_t np = p.items;  // items per pipeline window
     uint32_t* keys[2] = {at<uint32_t>(workspace, p.off_keys0), at<uint32_t>(workspace, p.off_keys1)};
     uint32_t* vals[2] = {at<uint32_t>(workspace, p.off_vals0), at<uint32_t>(workspace, p.off_vals1)};
-    k_digits<<<grid_for(n, 256), 256, 0, s>>>(reinterpret_cast<const uint4*>(scalars), n, p.c, p.Wd,
-                                              p.sgn, p.user_bits, p.glv, keys[0], status);
+    const PieceArgs pieces = piece_args(p, workspace, 0);
+    k_digits<<<grid_for(n, kDigitThreads), kDigitThreads, 0, s>>>(
+        reinterpret_cast<const uint4*>(scalars), n, p.c, p.Wd, p.sgn, p.user_bits, p.glv, keys[0], status,
+        pieces.nonzero ? pieces.ctrl + kNonzero : nullptr);
     note_launches(1);
     int cur = 0;
     bool pieces_counted = false;
@@ -2426,10 +2495,9 @@ int enqueue_head(const Plan& p, const uint32_t* points, const uint32_t* scalars,
                                               (int)kTileSmemMax));
             k_tile_count<<<dim3(p.ttiles, (unsigned)p.W), kTileThreads, smem, s>>>(keys[0], np, nb, p.tT, p.ttiles,
                                                                                   tcnt, rank);
-            const PieceArgs a = piece_args(p, workspace, 0);
             pieces_counted = p.ngroups == 1;
             k_tile_totals<<<grid_for(p.nbins, kBinBlock), kBinBlock, 0, s>>>(
-                tcnt, nb, p.ttiles, (uint32_t)p.W, bins, bsum, a.cap, pieces_counted ? a.ctrl + kHist : nullptr);
+                tcnt, nb, p.ttiles, (uint32_t)p.W, bins, bsum, pieces, pieces_counted ? 1 : 0);
             k_tile_offsets<<<grid_for(p.nbins, 256), 256, 0, s>>>(tcnt, nb, p.ttiles, (uint32_t)p.W, bins, bsum);
             k_tile_scatter<<<gw, 256, 0, s>>>(keys[0], rank, vals[0], total, np, nb, p.tT, p.ttiles, tcnt, p.np, pre_w);
             note_launches(4);
@@ -2481,10 +2549,8 @@ template <class M>
 int enqueue_group_tail_m(const Plan& p, const AccArgs& acc, int g, void* workspace, cudaStream_t s) {
     int* S = at<int>(workspace, p.off_S);
     const PieceArgs a = piece_args(p, workspace, g);
-    // 5. the parts of buckets cut into pieces, as many tree levels as a bucket can need
-    const size_t most = (p.items + p.K - 1) / p.K;   // pieces of one bucket
-    size_t per = 1;
-    for (int lv = 0; lv < 3 && most > per; ++lv, per *= kTreeParts) {
+    // 5. the parts of buckets cut into pieces
+    for (int lv = 0; lv < p.levels; ++lv) {
         const size_t want = p.max_tree[lv] + (lv == 0 ? (p.max_small + kTreeThreads - 1) / kTreeThreads : 0);
         k_merge_parts<M><<<(unsigned)(want < kTreeWave ? want : kTreeWave), kTreeThreads, 0, s>>>(
             acc.parts, acc.buckets, a.tree[lv], a.ctrl + kNTree + lv, lv == 0 ? a.small : nullptr,
