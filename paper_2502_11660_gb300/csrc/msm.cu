@@ -2150,7 +2150,23 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool single = true, size_t 
         // With many buckets the threads' sequential sums fill the GPU; few buckets' parts
         // go to blocks (816 buckets of 8 parts, XYZZ: 195 us by blocks, 280 us by threads).
         p->small_parts = nbk >= 2048 ? 8 : 2;
-        p->max_tree[0] = multi / (p->small_parts + 1) + 1;
+        // An installed K may cut most buckets into more parts than that: then the longest
+        // buckets' additions in sequence on one thread, half as many again as the mean's, against
+        // a block for every kTreeParts parts of a bucket (times of one addition as in the bucket
+        // reduction below). K = 2, n = 2^20, c = 16: XYZZ 102.2 -> 17.0, Edwards + GLV
+        // 21.0 -> 8.7 ms.
+        const size_t parts = (mean + K - 1) / K;
+        if (tk > 0 && nbk >= 2048 && parts >= p->small_parts) {
+            const double full = (double)nbk / (double)kWave;
+            const double t1 = p->edw ? std::max(10.5, 25.0 * full) : std::max(18.0, 29.0 * full);
+            const size_t of_block = std::min<size_t>(parts, kTreeParts);
+            const size_t blocks = nbk * ((parts + kTreeParts - 1) / kTreeParts), steps = (of_block + kTreeGroups - 1) / kTreeGroups + 4;
+            const double t4 = (p->edw ? 7.5 : 24.0) * (double)blocks / (double)kTreeWave;
+            if (1.5 * (double)parts * t1 < (double)steps * t4) p->small_parts = (uint32_t)(2 * parts);
+        }
+        // a bucket of more than small_parts parts has an entry for each kTreeParts of them: at
+        // most a 32nd of its parts, or one
+        p->max_tree[0] = multi / std::min<size_t>(p->small_parts + 1, kTreeParts / 2) + 1;
         p->max_tree[1] = p->max_tree[2] = multi / kTreeParts + 1;
         if (p->max_parts >= kPart || p->max_pieces >= (1ull << 32)) return false;
     }
