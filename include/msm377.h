@@ -212,7 +212,10 @@ typedef struct msm_opts {
     void *stream;          /* cudaStream_t */
 } msm_opts;
 
-/* Workspace bytes msm_g1 needs for n points with these options (0 on bad options). */
+/* Workspace bytes msm_g1 needs for n points with these options (0 on bad options). The
+ * need does not grow with n throughout (a larger n may take longer pieces of the bucket
+ * runs, and fewer of them): a workspace for calls of several sizes takes the largest of
+ * their needs. A call is refused (MSM377_ENOMEM) only where its own layout does not fit. */
 size_t msm_g1_workspace_bytes(size_t n, const msm_opts *opts);
 
 /* Window width msm_g1 uses for n points when opts.c == 0 (flags: the options'

@@ -39,6 +39,10 @@ int launch_validate(const uint32_t* points_std, size_t n, bool subgroup, int* st
 int msm_g1_run(const uint32_t* points, const uint32_t* scalars, size_t n, uint32_t* out, void* workspace,
                size_t workspace_bytes, const msm_opts* opts, bool overlap);
 
+// The bytes that one such call lays out (0 on bad options); msm_g1_workspace_bytes may ask
+// for more, so that a workspace serves smaller calls too.
+size_t msm_g1_layout_bytes(size_t n, const msm_opts* opts);
+
 inline unsigned grid_for(size_t n, unsigned block) {
     return static_cast<unsigned>((n + block - 1) / block);
 }

@@ -55,13 +55,13 @@ extern "C" int msm_g1_noalloc(const uint32_t* points, const uint32_t* scalars, s
     if (opts->flags & (MSM377_PROFILE | MSM377_VALIDATE))
         return set_error(MSM377_EINVAL, "msm_g1_noalloc: MSM377_PROFILE and MSM377_VALIDATE are not available on "
                          "this entry point (it reports no device status)");
-    size_t need = msm_g1_workspace_bytes(n, opts);
+    size_t need = msm_g1_layout_bytes(n, opts);
     msm_opts narrow = *opts;
     if (need > (size_t)MSM377_NOALLOC_SCRATCH_BYTES && opts->c == 0) {
         // The default width is the fastest one; a narrower one needs fewer buckets.
         for (int c = msm_g1_default_c(n, opts->signed_digits, opts->flags) - 1; c >= 4; --c) {
             narrow.c = c;
-            const size_t b = msm_g1_workspace_bytes(n, &narrow);
+            const size_t b = msm_g1_layout_bytes(n, &narrow);
             if (b != 0 && b <= (size_t)MSM377_NOALLOC_SCRATCH_BYTES) {
                 need = b;
                 opts = &narrow;

@@ -260,10 +260,15 @@ extern "C" int msm_g1_resident(msm_points_t handle, size_t offset, size_t n, con
     return msm_g1(msm_points_data(handle, offset), scalars, n, out, workspace, workspace_bytes, &o);
 }
 
+namespace {
+// A layout of `core` bytes with the copied scalars and the result behind it.
+size_t resident_host_bytes(size_t core, size_t n) { return align_up(core, 256) + align_up(n * 32, 256) + 256; }
+}  // namespace
+
 extern "C" size_t msm_g1_resident_host_workspace_bytes(msm_points_t handle, size_t n, const msm_opts* opts) {
     const size_t core = msm_g1_resident_workspace_bytes(handle, n, opts);
     if (!core) return 0;
-    return align_up(core, 256) + align_up(n * 32, 256) + 256;
+    return resident_host_bytes(core, n);
 }
 
 extern "C" int msm_g1_resident_host(msm_points_t handle, size_t offset, size_t n, const uint32_t* scalars_host,
@@ -274,12 +279,14 @@ extern "C" int msm_g1_resident_host(msm_points_t handle, size_t offset, size_t n
     if (n && !scalars_host) return set_error(MSM377_EINVAL, "msm_g1_resident_host: scalars_host is NULL");
     if (opts->flags & MSM377_PROFILE)
         return set_error(MSM377_EINVAL, "msm_g1_resident_host: MSM377_PROFILE is not available here");
-    const size_t need = msm_g1_resident_host_workspace_bytes(handle, n, opts);
-    if (!need) return set_error(MSM377_EINVAL, "msm_g1_resident_host: bad options");
+    msm_opts o;
+    if (resident_opts(as_set(handle), opts, &o)) return MSM377_EINVAL;
+    const size_t layout = msm_g1_layout_bytes(n, &o);
+    if (!layout) return set_error(MSM377_EINVAL, "msm_g1_resident_host: bad options");
+    const size_t core = align_up(layout, 256), need = resident_host_bytes(core, n);
     if (workspace_bytes < need)
         return set_error(MSM377_ENOMEM, "msm_g1_resident_host: workspace %zu bytes, need %zu", workspace_bytes, need);
     if (!aligned(workspace, 256)) return set_error(MSM377_EINVAL, "msm_g1_resident_host: workspace not 256-byte aligned");
-    const size_t core = align_up(msm_g1_resident_workspace_bytes(handle, n, opts), 256);
     char* base = static_cast<char*>(workspace);
     uint32_t* d_sc = reinterpret_cast<uint32_t*>(base + core);
     uint32_t* d_out = reinterpret_cast<uint32_t*>(base + core + align_up(n * 32, 256));
