@@ -417,9 +417,13 @@ int msm_g1_host(const uint32_t *points_host, const uint32_t *scalars_host, size_
  * as msm_g1 but uses a fixed scratch array of MSM377_NOALLOC_SCRATCH_BYTES
  * (64 MiB) that the library holds on every GPU that loads it, until the process
  * exits; it calls no cudaMalloc, cudaFree or other allocating routine.
- * - Size limit: n and the options must need at most MSM377_NOALLOC_SCRATCH_BYTES
- *   of workspace (msm_g1_workspace_bytes); with the default options that holds
- *   up to n = 2^15. Larger requests fail with MSM377_EINVAL and a message.
+ * - Size limit: n and the options must fit MSM377_NOALLOC_SCRATCH_BYTES. With an
+ *   explicit c that is its workspace at that width. With c = 0 a request that does
+ *   not fit at the default width runs at the widest narrower one (4 bits or more)
+ *   that does: the result is the same and the call slower than msm_g1. Without
+ *   MSM377_RADIX_SORT every request of up to n = 2^16 points with c = 0 is
+ *   accepted, whatever the curve model, the digits and the form of the points.
+ *   Larger requests fail with MSM377_EINVAL and a message.
  * - The first call on each device (and in each CUDA context: a driver-API
  *   context, or the primary context again after cudaDeviceReset) looks up the
  *   scratch address (a one-time set-up there); make that first call before any
