@@ -64,13 +64,13 @@ __device__ const static int kFold[kLimbs][16] = {
     {-532, -10211328, -94317, -9693512, -37529123, 23347729, 24436378, -1791456, 63052212, -63093489, -39261606, -55568259, 22282005, 7709679, 0, 0},
     {-18350080, -532, 22931456, -94390, 9170288, 4401012, 5727111, -47837953, -19358532, 16665979, 43836029, -24924431, -56390796, 0, 0, 0},
 };
-// limbs of p, 16 p, and (all mod p) d 2^432 (Edwards d = k / 2), s 2^864, gamma 2^864, 2^864
+// limbs of p, 32 p, and (all mod p) d 2^432 (Edwards d = k / 2), s 2^864, gamma 2^864, 2^864
 __device__ const static int kP27[16] = {
     1, 18350080, 532, 111286272, 94389, 125047440, 129816715, 128490616,
     47837952, 19358532, 117551749, 90381698, 24924430, 56390796, 0, 0};
-__device__ const static int k16P[16] = {
-    16, 25165824, 8514, 35749888, 1510237, 121710848, 63801534, 42583951,
-    94318607, 41301061, 1779794, 103929902, 130355434, 96946370, 6, 0};
+__device__ const static int k32P[16] = {
+    32, 50331648, 17028, 71499776, 3020474, 109203968, 127603069, 85167902,
+    54419486, 82602123, 3559588, 73642076, 126493141, 59675013, 13, 0};
 __device__ const static int kD432[16] = {
     28739701, -62258772, -63384102, -61773890, 41397844, -52194151, -1628871, -33266492,
     -56125541, 23385514, -38434099, -52534755, 43501085, -23480652, 0, 0};
@@ -216,8 +216,9 @@ __device__ __forceinline__ int unpack(const uint32_t* w, int lane) {
     return (int)(__funnelshift_r(lo, hi, sh) & (uint32_t)kDigit);
 }
 
-// c / R times (the integer in limbs l[0..14], |value| < 16 p, plus add0) mod p, in
-// [0, 2p), on one thread: + 16 p, carries, packing, and one Montgomery product by c.
+// c / R times (the integer in limbs l[0..14], |value| < 17 p, plus add0) mod p, in
+// [0, 2p), on one thread: + 32 p, which keeps it positive and below 49 p < 2^384, carries,
+// packing, and one Montgomery product by c (49 p c / R + p < 2 p).
 __device__ __forceinline__ fq::fe to_fe_times(const int* l, int add0, const fq::fe& c) {
     uint32_t w[13];
 #pragma unroll
@@ -225,7 +226,7 @@ __device__ __forceinline__ fq::fe to_fe_times(const int* l, int add0, const fq::
     int64_t carry = add0;
 #pragma unroll
     for (int j = 0; j < kLimbs; ++j) {
-        carry += (int64_t)l[j] + k16P[j];
+        carry += (int64_t)l[j] + k32P[j];
         const uint64_t dig = (uint64_t)(carry & kDigit);
         carry >>= kBits;                              // arithmetic
         const int bit = kBits * j, i = bit >> 5, sh = bit & 31;
@@ -266,7 +267,8 @@ __device__ __forceinline__ void put_fe(const Group& g, int i, const fq::fe& a) {
 //
 // The inverse of z in [1, p) (12 words in shared memory) mod p, on one warp, by
 // Bernstein and Yang's division steps ("Fast constant-time gcd computation and
-// modular inversion", 2019) in the half-delta form: with (delta, f, g) from
+// modular inversion", 2019) in the form that starts at delta = 1/2, whose bound on the steps
+// is P. Wuille's (safegcd-bounds, 2021): with (delta, f, g) from
 // (1/2, p, z), a step replaces (f, g) by (g, (g - f)/2) and delta by 1 - delta when
 // delta > 0 and g is odd, and else (f, g) by (f, (g + (g mod 2) f)/2) and delta by
 // 1 + delta. 27 steps depend on the low 27 bits only: they run on one register each
@@ -274,8 +276,7 @@ __device__ __forceinline__ void put_fe(const Group& g, int i, const fq::fe& a) {
 // 2^27, which is then applied to f, g and, mod p, to d, e with f = d z, g = e z. One
 // division by 2^27 is one limb, so an application is two multiply-adds per lane and
 // the carry round of a product. At most floor((45907 * 377 + 26313) / 19929) = 869
-// steps bring g to 0 (the published bound for this form), 33 rounds of 27; measured
-// over random z: 27 to 29 rounds. Then f = +-1 and z^-1 = f d.
+// steps bring g to 0, 33 rounds of 27; measured over random z: 27 to 29 rounds. Then f = +-1 and z^-1 = f d.
 // About 20 us instead of 80 us for one thread's binary GCD (ec::inv).
 constexpr int kInvRounds = 33;
 
@@ -287,7 +288,9 @@ __device__ __forceinline__ int shift_round(int lane, int p, int a, int x, int b,
     return from_lane(digit0(s), lane + 1) + digit1(s) + from_lane(digit2(s), lane + 31);
 }
 
-// p: limb `lane` of p. Limb `lane` of the inverse (|value| < 16 p).
+// p: limb `lane` of p. Limb `lane` of the inverse. A round replaces d and e, 0 and 1 at
+// first, by (a d + b e + m p) / 2^27 with |a| + |b| <= 2^27 and |m| <= 2^26, so it adds at most
+// p / 2 to the larger of their magnitudes: after the 33 rounds |value| <= 16.5 p + 1.
 __device__ __forceinline__ int inverse(int lane, int p, const uint32_t* z) {
     int f = p, gg = unpack(z, lane), d = 0, e = lane == 0 ? 1 : 0;
     int delta2 = 1;                                    // 2 delta
