@@ -223,7 +223,8 @@ size_t msm_g1_workspace_bytes(size_t n, const msm_opts *opts);
 int msm_g1_default_c(size_t n, int signed_digits, uint32_t flags);
 
 /* Installs measured window widths for signed digits: c_by_log2n[k] is used for
- * n in [2^k, 2^(k+1)) when opts.c == 0 (0 keeps the built-in rule). One table per
+ * n in [2^k, 2^(k+1)) when opts.c == 0 (0 keeps the built-in rule), except by the jobs
+ * of msm_g1_batched, whose widths follow the jobs' sizes. One table per
  * combination of MSM377_EDWARDS, MSM377_GLV and MSM377_PRECOMPUTED, chosen by flags
  * (other bits: MSM377_EINVAL; with PRECOMPUTED the table only advises which c to
  * precompute for, since those calls need an explicit c). len <= 32; len = 0 clears that table. Process-wide; written by
@@ -238,7 +239,8 @@ int msm_g1_set_window_table(const int32_t *c_by_log2n, int len, uint32_t flags);
  * (window groups, 1..8: the accumulation runs group by group and each group's
  * merges and bucket reduction run on a high-priority helper stream of the caller's
  * stream, overlapping the next group's accumulation); 0 in a field keeps the
- * built-in rule. Process-wide, like the window tables (written by the autotuner);
+ * built-in rule. All but the sort are for calls of one MSM: msm_g1_batched keeps
+ * its own rules, which look at the whole batch. Process-wide, like the window tables (written by the autotuner);
  * workspace sizes depend on it, so install before sizing workspaces. */
 int msm_g1_set_schedule(uint32_t flags, int log2n, int c, int chunk, int sort, int reduce_log2, int groups);
 

@@ -2,8 +2,8 @@
 
 For each size n = 2^k it times msm_g1 on the device (resident prepared points,
 fresh scalars) for every candidate c, keeps the fastest, and installs the table
-into the library (msm_g1_set_window_table), so every later call with c = 0 --
-single, batched or served -- uses the measured choice. The library keeps one
+into the library (msm_g1_set_window_table), so every later call of one MSM with
+c = 0 uses the measured choice (a batch keeps the library's rules). The library keeps one
 table per curve model / GLV combination; tune and install the one you run.
 Tables can be saved to and loaded from a JSON file keyed by the device name.
 
@@ -93,7 +93,7 @@ def candidates(log2n: int, glv: bool = False, precomputed: bool = False) -> list
 # run-to-run spread of these timings on GB300: at n = 2^16, c = 12 and c = 16 came out
 # 0.4 % apart in one run and 1.4 % apart, either way, in two others), and the widest is
 # kept: fewer windows mean fewer mixed additions, which is what counts when several MSMs
-# share the GPU (batched calls, serving).
+# share the GPU (serving).
 C_TIE = 0.01
 
 

@@ -2000,10 +2000,12 @@ constexpr int8_t kDefaultC[4][kDefaultLogs] = {
 
 // single: one call on its own, whose latency counts. The jobs of a batch overlap, so their
 // total work counts, and there the rule by size below is the better one (24 jobs of 2^10
-// to 2^18 points: 7.25 ms, 7.33 with the table).
+// to 2^18 points: 7.25 ms, 7.33 with the table). Installed widths are measured on single calls
+// too and are not taken there either (30 jobs of 2^10 to 2^13 points, Edwards + GLV, in one
+// graph: 1964 us by the rule, 2354 with a tuned table; 24 of 2^10 to 2^18 8748 and 8930).
 int default_c(size_t n, int sgn, uint32_t flags, bool single = true) {
     int lg = n > 1 ? ilog2(n) : 0;
-    if (sgn && lg < 32) {
+    if (single && sgn && lg < 32) {
         const int t = g_ctable[table_mode(flags)][lg].load(std::memory_order_relaxed);
         if (t > 0) return t;
     }
@@ -2058,9 +2060,11 @@ bool make_plan(size_t n, const msm_opts* o, Plan* p, bool single = true, size_t 
     // stays available for comparison.
     const int lgn = n > 1 ? ilog2(n) : 0;
     const int tmode = table_mode(o->flags);
+    // installed entries measured on single calls rule these only (default_c); the sort is a
+    // choice for any call
     const int tsort = (p->sgn && lgn < 32) ? g_sorttable[tmode][lgn].load(std::memory_order_relaxed) : 0;
-    const int tk = (p->sgn && lgn < 32) ? g_ktable[tmode][lgn].load(std::memory_order_relaxed) : 0;
-    const int tr = (p->sgn && lgn < 32) ? g_rtable[tmode][lgn].load(std::memory_order_relaxed) : 0;
+    const int tk = (single && p->sgn && lgn < 32) ? g_ktable[tmode][lgn].load(std::memory_order_relaxed) : 0;
+    const int tr = (single && p->sgn && lgn < 32) ? g_rtable[tmode][lgn].load(std::memory_order_relaxed) : 0;
     const int tg = (p->sgn && lgn < 32) ? g_gtable[tmode][lgn].load(std::memory_order_relaxed) : 0;
     p->counting = ((o->flags & MSM377_RADIX_SORT) || tsort == 2) ? 0 : 1;
     p->tiles = (items + kSortTile - 1) / kSortTile;
