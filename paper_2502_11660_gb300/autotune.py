@@ -80,13 +80,21 @@ def time_msm(n: int, c: int, reps: int = 3, device="cuda", seed: int = 11, edwar
     return float(np.median(times))
 
 
-def candidates(log2n: int, glv: bool = False, precomputed: bool = False) -> list[int]:
+def candidates(log2n: int, glv: bool = False, precomputed: bool = False, edwards: bool = False) -> list[int]:
     """Window widths to time at n = 2^log2n: 12..17 for the large sizes (15..20 for
-    fixed-base sets); around the built-in rule below 2^16."""
+    fixed-base sets); below 2^16 those around log2(n) - 4 and, from 2^11 on, 11 (it divides the
+    scalars' bits well); always the width that msm_g1 takes now, so that tuning cannot
+    lose to it."""
     if log2n >= 16:
-        return list(PRECOMPUTED_C if precomputed else LARGE_C)
-    base = max(4, log2n - 4 + (1 if glv else 0))
-    return sorted({max(3, base - 2), max(3, base - 1), base, base + 1, base + 2})
+        cs = set(PRECOMPUTED_C if precomputed else LARGE_C)
+    else:
+        base = max(4, log2n - 4 + (1 if glv else 0))
+        cs = set(range(max(3, base - 2), base + (3 if precomputed else 4)))
+        if log2n >= 11 and not precomputed:
+            cs.add(11)
+    if not precomputed:
+        cs.add(msm_g1_default_c(1 << log2n, True, edwards, glv))
+    return sorted(cs)
 
 
 # Window widths timed within this fraction of the fastest count as a tie (about the
@@ -111,7 +119,7 @@ def tune(log2_sizes=range(10, 23, 2), reps: int = 3, device="cuda", edwards: boo
     for k in log2_sizes:
         n = 1 << k
         t = {c: time_msm(n, c, reps, device, edwards=edwards, glv=glv, precomputed=precomputed)
-             for c in candidates(k, glv, precomputed)}
+             for c in candidates(k, glv, precomputed, edwards)}
         timings[k] = t
         best[k] = pick_c(t)
     table = [0] * 32
@@ -155,7 +163,7 @@ def tune_schedule(log2_sizes=range(10, 23), reps: int = 3, device="cuda", edward
         cur = [0, 0, 0, 0, 0]
         rec = {}
         t = {c: time_schedule(n, c, 0, 0, 0, 0, reps, device, edwards=edwards, glv=glv)
-             for c in candidates(k, glv)}
+             for c in candidates(k, glv, edwards=edwards)}
         cur[0] = pick_c(t)
         rec["c"] = t
         for field, values in ((1, CHUNKS), (2, SORTS), (3, REDUCE_LOG2), (4, GROUPS)):
