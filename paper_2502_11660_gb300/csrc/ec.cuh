@@ -111,7 +111,9 @@ __device__ __forceinline__ void dbl(xyzz& P) {
 // madd_but_double leaves P = Q undone and returns true: the caller doubles Q.
 // kMerged: Y3's two products share one reduction (fq::mulsum): 2628 instead of 2760 limb
 // products, and one more function in the kernel. Bucket accumulation at n = 2^20: 5.56 ->
-// 5.29 ms; but padd_batch 459 -> 506 us, so it keeps the two products.
+// 5.29 ms. padd_batch has the two products: they were the faster form in a kernel that also
+// converted standard forms (459 us, merged 506; n = 1000003). In the present k_padd they take
+// 447 and the merged form 429.
 template <bool kMerged = true>
 __device__ __forceinline__ bool madd_but_double(xyzz& P, bool& p_inf, const affine& Q) {
     if (is_inf(Q)) return false;
@@ -153,11 +155,6 @@ __device__ __forceinline__ void madd(xyzz& P, bool& p_inf, const affine& Q) {
         mdbl(P, Q);
         p_inf = is_inf(P);
     }
-}
-
-__device__ __forceinline__ void madd(xyzz& P, const affine& Q) {
-    bool inf = is_inf(P);
-    madd(P, inf, Q);
 }
 
 // Second operand of add_q() held in registers.

@@ -1985,12 +1985,16 @@ int table_mode(uint32_t flags) {
 }
 
 // Window width by floor(log2 n) for signed digits, per mode (bit 0 Edwards, bit 1 GLV):
-// the fastest of the widths 4..17 measured on GB300 at 1.05 and 1.55 times each power of
-// two (the better of the two on average). A wider window means fewer windows but more
-// buckets; which widths pay also depends on the top window, which is short (and its
-// few buckets heavy) when c just fails to divide the scalar's bits: with GLV's 127-bit
-// halves 11 and 16 divide well, so n = 2^16 .. 2^22 takes 16 (n = 2.7 * 10^5, Edwards + GLV:
-// c = 14 1949, 15 1742, 16 1616, 17 1858 us) and 2^12 .. 2^14 takes 11.
+// the fastest of the widths 4..17 on GB300 at 1.05 and 1.55 times each power of two (the
+// better of the two on average). A wider window means fewer windows but more buckets; which
+// widths pay also depends on the top window, which is short (and its few buckets heavy) when
+// c just fails to divide the scalar's bits: with GLV's 127-bit halves 11 and 16 divide well, so
+// with Edwards + GLV 2^12 .. 2^14 takes 11 and 2^17 .. 2^22 16 (n = 2.7 * 10^5: c = 14 1965, 15 1721,
+// 16 1596, 17 1869 us). That sweep came before the merged Y3 of XYZZ additions, the two-lane
+// segment sums and the shorter pieces; measured again with them (widths 3..18, 2^4 .. 2^22), the
+// entries are within 2.1 % of the fastest width but for these: c = 8 at 2^4 and 2^5 is 2 to
+// 9 % faster in every mode; XYZZ 2^12: 11 5.5 %, 2^16: 14 3.6 %; GLV 2^20: 16 3.6 %, 2^21 and 2^22:
+// 18 2.7 and 5.0 %.
 constexpr int kDefaultLogs = 23;
 constexpr int8_t kDefaultC[4][kDefaultLogs] = {
     {4, 4, 4, 4, 4, 4, 6, 6, 7, 7, 8, 11, 8, 11, 11, 13, 13, 15, 15, 16, 16, 17, 17},   // XYZZ

@@ -348,8 +348,6 @@ __device__ __forceinline__ fq::fe inverse_fe(const fq::fe& a, int src, uint32_t*
 // ---------------------------------------------------------------- Edwards
 
 struct Edwards {
-    static constexpr int kCoords = 4;
-
     static __device__ __forceinline__ void set_inf(const Group& g) {   // (0 : 1 : 1 : 0)
         g.st(g.w, (g.w == Y || g.w == Z) && g.lane == 0 ? 1 : 0);
         __syncthreads();
@@ -481,8 +479,6 @@ struct Edwards {
 // ---------------------------------------------------------------- Weierstrass
 
 struct Weierstrass {
-    static constexpr int kCoords = 3;
-
     static __device__ __forceinline__ void set_inf(const Group& g) {   // (0 : 1 : 0)
         if (g.w < 3) g.st(g.w, g.w == Y && g.lane == 0 ? 1 : 0);
         __syncthreads();
