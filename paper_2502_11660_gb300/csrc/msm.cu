@@ -695,7 +695,8 @@ __global__ void __launch_bounds__(128, 3) k_precompute_ed(const uint4* __restric
 // Window digits of one scalar (8 words, little-endian) for point index `idx`:
 // |digit| (0 = no contribution) with its sign in bit 31, window-major ([W][np]). The
 // point of an item follows from its place (item_point), so it is not stored. Returns how
-// many digits are not zero.
+// many digits are not zero (kCount; else 0).
+template <bool kCount>
 __device__ __forceinline__ uint32_t emit_digits(const uint32_t (&s)[8], int c, int W, int sgn, size_t idx,
                                             size_t np, uint32_t* __restrict__ keys) {
     const uint32_t cmask = (1u << c) - 1u, half = 1u << (c - 1);
@@ -723,7 +724,7 @@ __device__ __forceinline__ uint32_t emit_digits(const uint32_t (&s)[8], int c, i
             key = raw;
         }
         keys[(size_t)j * np + idx] = key | (neg << 31);
-        nonzero += key != 0;
+        if (kCount) nonzero += key != 0;
     }
     return nonzero;
 }
@@ -842,7 +843,8 @@ __device__ __forceinline__ void glv_split(uint32_t (&k)[8], uint32_t (&k1)[8], u
     }
 }
 
-// The digits of scalar i; returns how many are not zero.
+// The digits of scalar i; returns how many are not zero (kCount; else 0).
+template <bool kCount>
 __device__ __forceinline__ uint32_t scalar_digits(const uint4* __restrict__ scalars, size_t i, size_t n, int c, int W, int sgn,
                                                   int bits, int glv, uint32_t* __restrict__ keys, int* __restrict__ status) {
     uint4 lo = scalars[2 * i], hi = scalars[2 * i + 1];
@@ -858,25 +860,26 @@ __device__ __forceinline__ uint32_t scalar_digits(const uint4* __restrict__ scal
         }
         if (over) atomicCAS(status, 0, MSM377_ERANGE);   // the first error of the call stays
     }
-    if (!glv) return emit_digits(s, c, W, sgn, i, n, keys);
+    if (!glv) return emit_digits<kCount>(s, c, W, sgn, i, n, keys);
     uint32_t k1[8], k2[8];
     glv_split(s, k1, k2);
-    const uint32_t m = emit_digits(k1, c, W, sgn, 2 * i, 2 * n, keys);     // P_i
-    return m + emit_digits(k2, c, W, sgn, 2 * i + 1, 2 * n, keys);         // phi(P_i)
+    const uint32_t m = emit_digits<kCount>(k1, c, W, sgn, 2 * i, 2 * n, keys);     // P_i
+    return m + emit_digits<kCount>(k2, c, W, sgn, 2 * i + 1, 2 * n, keys);         // phi(P_i)
 }
 
-// nonzero: the count of digits that are not zero is added there (null: not counted; see
-// piece_cap).
+// kCount: the count of digits that are not zero is added to *nonzero (piece_cap), 5 us at
+// n = 2^20; calls of short pieces, which do not ask for it, are spared 1 us of 8.
 constexpr int kDigitThreads = 256;
 
+template <bool kCount>
 __global__ void __launch_bounds__(kDigitThreads) k_digits(const uint4* __restrict__ scalars, size_t n, int c, int W, int sgn,
                                                           int bits, int glv, uint32_t* __restrict__ keys,
                                                           int* __restrict__ status, uint32_t* __restrict__ nonzero) {
     __shared__ uint32_t block_count;
-    if (threadIdx.x == 0) block_count = 0;
     const size_t i = blockIdx.x * (size_t)kDigitThreads + threadIdx.x;
-    uint32_t m = i < n ? scalar_digits(scalars, i, n, c, W, sgn, bits, glv, keys, status) : 0u;
-    if (!nonzero) return;   // the whole grid
+    uint32_t m = i < n ? scalar_digits<kCount>(scalars, i, n, c, W, sgn, bits, glv, keys, status) : 0u;
+    if (!kCount) return;
+    if (threadIdx.x == 0) block_count = 0;
     __syncthreads();
     m = __reduce_add_sync(0xffffffffu, m);
     if ((threadIdx.x & 31) == 0) atomicAdd(&block_count, m);
@@ -1451,8 +1454,9 @@ __device__ __forceinline__ uint32_t plan_merge(const PieceArgs& a, uint32_t np, 
         return base;
     }
     uint32_t src = base, cnt = np;
-    for (int lv = 0; lv < a.levels; ++lv) {
-        const uint32_t nout = lv + 1 == a.levels ? 1u : (cnt + kTreeParts - 1) / kTreeParts;
+#pragma unroll
+    for (int lv = 0; lv < 3; ++lv) {   // the last level has one output
+        const uint32_t nout = lv == 2 || lv + 1 == a.levels ? 1u : (cnt + kTreeParts - 1) / kTreeParts;
         const uint32_t e = atomicAdd(&a.ctrl[kNTree + lv], nout);
         if (nout == 1) {
             a.tree[lv][e] = make_uint4(src, cnt, bucket, 0u);
@@ -2513,9 +2517,10 @@ int enqueue_head(const Plan& p, const uint32_t* points, const uint32_t* scalars,
     uint32_t* keys[2] = {at<uint32_t>(workspace, p.off_keys0), at<uint32_t>(workspace, p.off_keys1)};
     uint32_t* vals[2] = {at<uint32_t>(workspace, p.off_vals0), at<uint32_t>(workspace, p.off_vals1)};
     const PieceArgs pieces = piece_args(p, workspace, 0);
-    k_digits<<<grid_for(n, kDigitThreads), kDigitThreads, 0, s>>>(
-        reinterpret_cast<const uint4*>(scalars), n, p.c, p.Wd, p.sgn, p.user_bits, p.glv, keys[0], status,
-        pieces.nonzero ? pieces.ctrl + kNonzero : nullptr);
+    const auto digits = pieces.nonzero ? k_digits<true> : k_digits<false>;
+    digits<<<grid_for(n, kDigitThreads), kDigitThreads, 0, s>>>(reinterpret_cast<const uint4*>(scalars), n, p.c, p.Wd,
+                                                                p.sgn, p.user_bits, p.glv, keys[0], status,
+                                                                pieces.ctrl + kNonzero);
     note_launches(1);
     int cur = 0;
     bool pieces_counted = false;
